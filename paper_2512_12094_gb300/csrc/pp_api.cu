@@ -1695,7 +1695,7 @@ pp_status pp_expect(pp_ctx* c, const double* bloch, double* out) {
     std::vector<double> bv(bloch, bloch + 3 * n);
     if (bv != c->sn_bloch) {
       PP_CUDA(launch_sn_table(n, c->stream, c->d_bloch, c->d_sn_work, c->d_sn));
-      c->launches += 1;
+      c->launches += n;
       c->sn_bloch = bv;
     }
     a.sn_table = c->d_sn;

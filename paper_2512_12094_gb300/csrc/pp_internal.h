@@ -202,8 +202,9 @@ cudaError_t launch_overlap(int W, int grid, cudaStream_t s, const uint64_t* keys
                            const unsigned long long* count_dev, const OverlapArgs& a,
                            double* partials, double* out);
 
-// S_n orbit-averaged overlap table [(n+1)^3] for a product state (one block);
-// work is a scratch buffer of the same size.
+// S_n orbit-averaged overlap table [(n+1)^3] for a product state (n launches;
+// entries with x + y + z > n are left as they are); work is a scratch buffer of
+// the same size.
 cudaError_t launch_sn_table(int n, cudaStream_t s, const double* bloch, double* work,
                             double* table);
 

@@ -19,6 +19,8 @@
 // races with another insert of the same key.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "pp_device.cuh"
 
 namespace cg = cooperative_groups;
@@ -856,36 +858,30 @@ __global__ void __launch_bounds__(kBlock) reduce_partials_kernel(const double* p
 // sites are filled in order, site k drawing each remaining letter with
 // probability (remaining count) / (remaining sites).  E_k over states
 // (x, y, z) of remaining counts; every step is a convex combination.
-__global__ void __launch_bounds__(1024) sn_table_kernel(int n, const double* bloch, double* table,
-                                                       double* work) {
-  const int S = n + 1;
-  const size_t total = (size_t)S * S * S;
-  // after n steps the result must sit in `table`: start in whichever buffer
-  // makes the last write land there
-  double* nxt = (n & 1) ? work : table;
-  double* cur = (n & 1) ? table : work;
-  for (size_t i = threadIdx.x; i < total; i += blockDim.x) nxt[i] = (i == 0) ? 1.0 : 0.0;
-  __syncthreads();
-  for (int k = n - 1; k >= 0; --k) {
-    const int left = n - k;
-    const double bX = bloch[3 * k], bY = bloch[3 * k + 1], bZ = bloch[3 * k + 2];
-    for (size_t f = threadIdx.x; f < total; f += blockDim.x) {
-      const int z = (int)(f % S), y = (int)((f / S) % S), x = (int)(f / ((size_t)S * S));
-      double v = 0.0;
-      if (x + y + z <= left) {
-        const int iI = left - x - y - z;
-        if (iI > 0) v += (double)iI * nxt[f];
-        if (x > 0) v += (double)x * bX * nxt[f - (size_t)S * S];
-        if (y > 0) v += (double)y * bY * nxt[f - S];
-        if (z > 0) v += (double)z * bZ * nxt[f - 1];
-        v /= (double)left;
-      }
-      cur[f] = v;
-    }
-    __syncthreads();
-    double* tmp = cur;
-    cur = nxt;
-    nxt = tmp;
+//
+// One launch per site: block (x, y), one thread per z.  Only the states that
+// fit the `left` sites still open, x + y + z <= left, are computed; a step
+// reads none but those of the step before it, so nothing else needs a value.
+// Bound by the chain of n launches (n = 64: 0.17 ms, 16.4 ms when one block
+// filled the whole (n + 1)^3 cube at every site).
+__global__ void __launch_bounds__(kBlock)
+    sn_table_step_kernel(int n, int k, const double* __restrict__ bloch,
+                         const double* __restrict__ nxt, double* __restrict__ cur) {
+  const int S = n + 1, left = n - k;
+  const int x = blockIdx.x, y = blockIdx.y;
+  const double bX = bloch[3 * k], bY = bloch[3 * k + 1], bZ = bloch[3 * k + 2];
+  for (int z = threadIdx.x; x + y + z <= left; z += blockDim.x) {
+    const size_t f = ((size_t)x * S + y) * S + z;
+    // before the last site only the empty state is left, with value 1
+    auto at = [&](size_t i) { return left == 1 ? 1.0 : nxt[i]; };
+    double v = 0.0;
+    const int iI = left - x - y - z;
+    if (iI > 0) v += (double)iI * at(f);
+    if (x > 0) v += (double)x * bX * at(f - (size_t)S * S);
+    if (y > 0) v += (double)y * bY * at(f - S);
+    if (z > 0) v += (double)z * bZ * at(f - 1);
+    v /= (double)left;
+    cur[f] = v;
   }
 }
 
@@ -1115,7 +1111,14 @@ cudaError_t launch_overlap(int W, int grid, cudaStream_t s, const uint64_t* keys
 
 cudaError_t launch_sn_table(int n, cudaStream_t s, const double* bloch, double* work,
                             double* table) {
-  sn_table_kernel<<<1, 1024, 0, s>>>(n, bloch, table, work);
+  // the last step (k = 0) writes `table`
+  for (int k = n - 1; k >= 0; --k) {
+    const int left = n - k;
+    double* cur = (k & 1) ? work : table;
+    const double* nxt = (k & 1) ? table : work;
+    const int threads = std::min(kBlock, (left + 32) / 32 * 32);
+    sn_table_step_kernel<<<dim3(left + 1, left + 1), threads, 0, s>>>(n, k, bloch, nxt, cur);
+  }
   return cudaGetLastError();
 }
 
