@@ -24,6 +24,7 @@
 
 #include "../../include/pp.h"
 #include "pp_internal.h"
+#include "pp_phase.h"
 #include "pp_symmetry_host.h"
 
 using namespace ppk;
@@ -93,6 +94,9 @@ struct ArgsEntry {
   GateArgs* d_args = nullptr;      // device copy
   size_t n = 0;                    // its size in bytes
   uint64_t last_use = 0;
+  // mean number of live strings of a gate's table that anticommuted with it in
+  // the last layer, per gate (apply_layer_phased)
+  std::vector<float> activity;
 };
 
 struct GraphEntry {
@@ -108,6 +112,18 @@ size_t table_bytes(uint64_t cap, uint64_t icap, int W, size_t row_bytes) {
   return (size_t)cap * (16 * W + row_bytes) + (size_t)icap * 8;
 }
 
+}  // namespace
+
+namespace {
+// Mean number of gates of a phase that may be active on a string.  More mean
+// fewer phases, two passes over the table each, but larger classes; one that
+// outgrows a block sends the layer back.  Measured (layers of the n = 32 ring,
+// plain / merged, and of the 5 x 6 torus, ms): limit 2: 4.6 / 23.8 / 40.3, 3:
+// 4.4 / 18.5 / 38.9, 5: 3.9 / 16.9 / 37.9, 9: 3.9 / 18.0 / 64.5 (torus layers
+// given up).
+constexpr double kPhaseActive = 5.0;
+constexpr float kPhaseGuess = 0.09f;  // a gate's mean activity while nothing is known
+constexpr int kActivityMax = 8192;
 }  // namespace
 
 struct pp_ctx {
@@ -161,6 +177,14 @@ struct pp_ctx {
   double grid_frac = 1.0;    // a persistent layer launch takes at most this fraction of the GPU
   double gate_ms = 0.0;
   int64_t gates_timed = 0;
+  bool index_ok = true;        // the active table's index and occupancy masks are valid
+  bool phase_off = false;      // pp_tune chose the persistent kernel for this context
+  double phase_active = kPhaseActive;  // limit on the mean number of active gates of a phase
+  double phase_room = 1.0;     // buckets per layer relative to the default sizing
+  int phase_wait = 0;          // layers left before phases are tried again
+  int phase_fails = 0;         // phased layers given up in a row
+  int phase_gates = kPhaseGates;  // of a phase at most
+  float* h_activity = nullptr; // pinned, kActivityMax gates
   void* sort_scratch = nullptr;  // scratch of the sort-based merge (merge_method 1)
   size_t sort_scratch_bytes = 0;
 };
@@ -428,6 +452,7 @@ pp_status compact_into(pp_ctx* c, int dst, double extra_eps, int extra_wmax) {
     PP_TRY(ctl_commit(c));
   }
   PP_TRY(activate(c, dst));
+  c->index_ok = true;
   c->compactions++;
   return PP_OK;
 }
@@ -556,6 +581,7 @@ pp_status merge_active(pp_ctx* c, int group) {
   c->launches += 2;
   PP_TRY(ctl_commit(c));
   PP_TRY(activate(c, dst));
+  c->index_ok = true;
   c->merged = true;
   c->merges++;
   return PP_OK;
@@ -566,11 +592,10 @@ pp_status merge_active(pp_ctx* c, int group) {
 // on the device and does nothing if a gate stopped for capacity.  The host
 // reads the control block once afterwards (finish_queued_merge) instead of
 // once after the gates and once after the merge.
-pp_status queue_merge(pp_ctx* c, int group) {
+pp_status queue_merge(pp_ctx* c, int group, int src, int dst) {
   Range range_("queue merge");
-  const int dst = 1 - c->active;
   Buf& d = c->buf[dst];
-  Buf& s = c->buf[c->active];
+  Buf& s = c->buf[src];
   PP_CUDA(cudaMemsetAsync(d.index, 0, (size_t)d.icap * 8, c->stream));
   PP_CUDA(launch_ctl_insert(c->stream, c->d_ctl, 0, 1));
   const int grid = c->sms * 8;  // grid-stride; the count is on the device
@@ -591,12 +616,14 @@ pp_status queue_merge(pp_ctx* c, int group) {
   return PP_OK;
 }
 
-// After the control block was read and showed no stall: the queued merge ran.
-pp_status finish_queued_merge(pp_ctx* c) {
+// After the control block was read and showed no stall: the queued merge into
+// table dst ran.
+pp_status finish_queued_merge(pp_ctx* c, int dst) {
   c->n_terms = c->h_ctl->n_terms;
   c->n_live = c->h_ctl->n_live;
   c->live_known = true;
-  PP_TRY(activate(c, 1 - c->active));
+  if (dst != c->active) PP_TRY(activate(c, dst));
+  c->index_ok = true;
   c->merged = true;
   c->merges++;
   return PP_OK;
@@ -764,6 +791,7 @@ pp_status ingest_terms(pp_ctx* c, int64_t n_terms, const uint64_t* x, const uint
     if ((st = ctl_commit(c)) != PP_OK) return release(st);
     release(PP_OK);
   }
+  c->index_ok = true;
   c->merged = true;
   return PP_OK;
 }
@@ -1063,14 +1091,14 @@ pp_status collect_gate_times(pp_ctx* c, unsigned from, unsigned to) {
 }
 
 // Device copy of a layer's gate arguments (cached by content).
-pp_status device_args(pp_ctx* c, const std::vector<GateArgs>& args, const GateArgs** out) {
+pp_status device_args(pp_ctx* c, const std::vector<GateArgs>& args, ArgsEntry** out) {
   std::vector<unsigned char> sig(args.size() * sizeof(GateArgs));
   memcpy(sig.data(), args.data(), sig.size());
   c->graph_clock++;
   for (auto& e : c->arg_cache) {
     if (e.sig == sig) {
       e.last_use = c->graph_clock;
-      *out = e.d_args;
+      *out = &e;
       return PP_OK;
     }
   }
@@ -1088,8 +1116,8 @@ pp_status device_args(pp_ctx* c, const std::vector<GateArgs>& args, const GateAr
   PP_CUDA(upload(c, ent.d_args, args.data(), ent.n));
   ent.sig = std::move(sig);
   ent.last_use = c->graph_clock;
-  *out = ent.d_args;
   c->arg_cache.push_back(std::move(ent));
+  *out = &c->arg_cache.back();
   return PP_OK;
 }
 
@@ -1154,6 +1182,7 @@ pp_status restore_snapshot(pp_ctx* c, const Buf& s, uint64_t n) {
   }
   PP_TRY(ctl_commit(c));
   PP_TRY(activate(c, c->active));
+  c->index_ok = true;
   c->merged = true;
   return PP_OK;
 }
@@ -1165,11 +1194,240 @@ pp_status restore_snapshot(pp_ctx* c, const Buf& s, uint64_t n) {
 uint64_t layer_grid_want(const pp_ctx* c, uint64_t n_now) {
   const int nt = c->batched ? kBlock : c->layer_threads;
   const uint64_t rowf = c->batched ? std::max<uint64_t>(1, (uint64_t)c->B / 32) : 1;
-  const double grow = c->batched ? std::max(1.25, c->last_growth) : 1.25;
+  // a layer that multiplied the table (an all-to-all layer merged under S_n
+  // starts from a handful of representatives) is sized for what it grew to
+  const double grow = (c->batched || c->last_growth > 8.0) ? std::max(1.25, c->last_growth) : 1.25;
   const double e = std::max(1.0, (double)n_now * grow);
   const uint64_t want = (uint64_t)std::ceil(e * (double)rowf * c->grid_scale / nt);
   const uint64_t full = std::max<uint64_t>(1, (uint64_t)c->sms * c->layer_bps);
   return std::min<uint64_t>(std::max<uint64_t>(want, 1), full);
+}
+
+// Phases take the place of the persistent layer kernel on single FP64 columns.
+// A caller that sets the block size of that kernel, or the limit of the waits
+// at its barriers, asks for it; pp_tune may have measured it faster.
+bool phases_allowed(const pp_ctx* c) {
+  return !c->batched && c->cfg.block_threads == 0 && c->cfg.wait_limit == 0 && !c->phase_off;
+}
+
+// Apply the layer as phases (pp_phase.cu) and, with merge, its symmetry merge.
+// *done is false when the layer does not suit them or had to be given up; the
+// table is then as it was, and the caller applies the layer the other way.
+//
+// Rule: at least kPhaseMinGates gates that touch a string per phase, since a phase
+// costs two passes over the table and two launches whatever it holds, and a
+// pass per gate costs one and a barrier.
+constexpr int kPhaseMinGates = 3;
+constexpr int kPhaseMax = 64;       // phases of a layer
+constexpr double kDenseFill = 700.0; // strings of a bucket in the expected table, dense classes
+constexpr int kPhaseBits = 10;      // key bits a run that does not commute may touch
+
+constexpr size_t kPhaseBytesMax = (size_t)64 << 30;
+
+size_t align256(size_t b) { return (b + 255) / 256 * 256; }
+
+// Dense classes (pp_phase.cu): one or two words, truncation on, no damping per
+// gate (which changes strings that a gate commutes with).
+bool dense_classes(const pp_ctx* c) {
+  return c->n <= 64 && c->cfg.coeff_eps > 0.0 && c->cfg.noise_mode != PP_NOISE_PER_GATE;
+}
+
+// Buckets of a phased layer of G gates in P phases, and its scratch.  One bucket
+// per resident warp (dense: block) at least, and enough that a bucket of the
+// expected table fills half a warp's room (dense: kDenseFill strings of the
+// block's 1024; 500 measured 1 to 6 % slower, 1200 the same).  A bucket has room
+// for four times that and more, since classes come in lumps.
+struct PhaseSizes {
+  double est;  // strings expected at the layer's end
+  uint64_t nb, cg;
+  size_t clear, bytes;
+};
+
+PhaseSizes phase_sizes(const pp_ctx* c, size_t G, size_t P) {
+  PhaseSizes z;
+  const int P32 = phase_words(c->n);
+  const bool dense = dense_classes(c);
+  z.est = (double)c->n_terms * std::max(1.5, 1.25 * c->last_growth);
+  const double half = dense ? kDenseFill : 0.5 * phase_strings_per_warp(P32);
+  const uint64_t least = (uint64_t)c->sms * (dense ? 2 : phase_warps_per_sm());
+  z.nb = std::max<uint64_t>(least, (uint64_t)std::ceil(z.est * c->phase_room / half));
+  z.cg = (256 + (uint64_t)(4.0 * z.est / (double)z.nb)) / 8 * 8;
+  z.clear = sizeof(PhaseStat) + G * 24 + P * z.nb * 4;
+  z.bytes = align256(z.clear) + align256(G * 4) +
+            2 * (align256(z.nb * z.cg * 8 * P32) + 2 * align256(z.nb * z.cg * 8));
+  return z;
+}
+
+pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateArgs>& args, bool merge,
+                             bool* done) {
+  *done = false;
+  const size_t G = args.size();
+  const uint64_t T = c->n_terms;
+  if (T == 0) return PP_OK;
+  if (c->phase_wait > 0) {
+    c->phase_wait--;
+    return PP_OK;
+  }
+  std::vector<ppphase::Gen> gens(G);
+  for (size_t g = 0; g < G; ++g) gens[g] = {args[g].px, args[g].pz};
+  // the control block read last holds the occupancy masks of this table (or,
+  // after a compaction, of a larger one)
+  static_assert(sizeof(c->h_ctl->occ[0]) == sizeof(uint64_t), "occupancy words");
+  uint64_t occ[2 * kMaxW];
+  for (int j = 0; j < 2 * kMaxW; ++j) occ[j] = c->h_ctl->occ[j];
+  const std::vector<unsigned char> touch =
+      ppphase::touched(gens, c->W, occ, occ + kMaxW, args[0].damp != nullptr);
+  const size_t n_touch = (size_t)std::count(touch.begin(), touch.end(), (unsigned char)1);
+  if (ent.activity.size() != G) ent.activity.assign(G, kPhaseGuess);
+  const bool dense = dense_classes(c);
+  ppphase::Limits lim;
+  lim.max_gates = c->phase_gates;
+  lim.max_active = c->phase_active;
+  lim.max_bits = kPhaseBits;
+  lim.triangular = dense;
+  const std::vector<ppphase::Phase> phases =
+      ppphase::plan(gens, c->W, touch.data(), ent.activity.data(), lim);
+  const size_t P = phases.size();
+  if (P == 0 || P > (size_t)kPhaseMax || P * kPhaseMinGates > n_touch) return PP_OK;
+  Range range_("phases");
+  const PhaseSizes z = phase_sizes(c, G, P);
+  const uint64_t nb = z.nb, cg = z.cg;
+  const size_t need = z.bytes;
+  const double est = z.est;
+  const int P32 = phase_words(c->n);
+  const int warps = std::max(4, (int)std::floor(c->sms * phase_warps_per_sm() * c->grid_frac));
+  auto al = align256;
+  const size_t clear = z.clear;
+  if (nb >= (1ull << 26) || need > kPhaseBytesMax) return PP_OK;
+  if (c->cfg.mem_budget_bytes && c->bytes + need > c->cfg.mem_budget_bytes) return PP_OK;
+  unsigned char* scratch = nullptr;
+  if (dmalloc(c, (void**)&scratch, need) != PP_OK) {  // no room for it: the other path
+    cudaGetLastError();
+    return PP_OK;
+  }
+  auto release = [&](pp_status st) {
+    dfree(c, scratch, need);
+    return st;
+  };
+  PhaseAcc acc;
+  acc.st = reinterpret_cast<PhaseStat*>(scratch);
+  acc.delta = reinterpret_cast<long long*>(acc.st + 1);
+  acc.ac = reinterpret_cast<unsigned long long*>(acc.delta + G);
+  acc.touch = reinterpret_cast<unsigned*>(acc.ac + G);
+  acc.seen = acc.touch + G;
+  unsigned* cnt = acc.seen + G;
+  acc.activity = reinterpret_cast<float*>(scratch + al(clear));
+  PhaseBuckets buckets[2];
+  {
+    unsigned char* p = scratch + al(clear) + al(G * 4);
+    for (int k = 0; k < 2; ++k) {
+      buckets[k].keys = reinterpret_cast<uint32_t*>(p);
+      p += al(nb * cg * 8 * P32);
+      buckets[k].coef = reinterpret_cast<double*>(p);
+      p += al(nb * cg * 8);
+      buckets[k].meta = reinterpret_cast<uint2*>(p);
+      p += al(nb * cg * 8);
+      buckets[k].cnt = nullptr;
+    }
+  }
+  std::vector<int> skip_after(G + 1, 0);  // gates from g on that touch nothing
+  for (size_t g = G; g-- > 0;) skip_after[g] = skip_after[g + 1] + !touch[g];
+  auto desc = [&](size_t p) {
+    PhaseDesc d;
+    memset(&d, 0, sizeof(d));
+    if (p < P) {
+      const ppphase::Phase& ph = phases[p];
+      d.first = ph.first;
+      d.count = ph.count;
+      d.commuting = ph.commuting;
+      d.dense = ph.triangular;
+      for (int k = 0; k < ph.count; ++k) d.skip |= (unsigned)!touch[ph.first + k] << k;
+      d.after = (int)G - ph.first - ph.count;
+      d.skip_after = skip_after[ph.first + ph.count];
+      memcpy(d.ux, ph.ux, sizeof(d.ux));
+      memcpy(d.uz, ph.uz, sizeof(d.uz));
+    }
+    return d;
+  };
+  PhaseRule rule;
+  rule.use_eps = args[0].use_eps;
+  rule.eps_bits = args[0].eps_bits;
+  rule.wmax = args[0].wmax;
+  rule.damp = args[0].damp;
+  const int src = c->active, dst = 1 - c->active;
+  cudaError_t e = cudaSuccess;
+  auto run = [&](cudaError_t r) { e = (e == cudaSuccess) ? r : e; };
+  if (c->cfg.profile_kernels) run(cudaEventRecord(c->ev_layer[0], c->stream));
+  run(launch_phase_begin(c->stream, acc, clear, c->d_ctl, c->sms));
+  buckets[0].cnt = cnt;
+  const int dgrid = (int)std::min<uint64_t>((T + kBlock - 1) / kBlock, (uint64_t)c->sms * 8);
+  run(launch_phase_deal(P32, dgrid, c->stream, desc_of(c, c->buf[src]), T, rule.use_eps, buckets[0],
+                        (unsigned)nb, (unsigned)cg, desc(0), ent.d_args, acc));
+  for (size_t p = 0; p < P; ++p) {
+    PhaseBuckets in = buckets[p & 1], out = buckets[(p + 1) & 1];
+    in.cnt = cnt + p * nb;
+    out.cnt = p + 1 < P ? cnt + (p + 1) * nb : nullptr;
+    run(launch_phase(P32, warps, c->stream, in, out, (unsigned)nb, (unsigned)cg, desc(p), desc(p + 1),
+                     ent.d_args, rule, desc_of(c, c->buf[dst]), c->d_ctl, acc));
+  }
+  run(launch_phase_end(c->stream, c->d_ctl, acc, (unsigned)G));
+  if (c->cfg.profile_kernels) run(cudaEventRecord(c->ev_layer[1], c->stream));
+  c->launches += (int64_t)P + 3;
+  if (e != cudaSuccess) return release(cuda_fail(e, "phase launch"));
+  c->index_ok = false;  // of either table from here on, until the merge has rebuilt one
+  if (merge) {
+    const pp_status st = queue_merge(c, c->cfg.symmetry, dst, src);
+    if (st != PP_OK) return release(st);
+  }
+  // per-gate activity, for the next plan of this layer; small tables need none
+  const bool want_activity = est >= 16384.0 && G <= (size_t)kActivityMax;
+  if (want_activity) {
+    if (!c->h_activity && pinned_get((void**)&c->h_activity, kActivityMax * sizeof(float)) != cudaSuccess)
+      return release(fail(PP_ERR_OOM, "pinned host allocation failed"));
+    run(cudaMemcpyAsync(c->h_activity, acc.activity, G * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
+    if (e != cudaSuccess) return release(cuda_fail(e, "activity download"));
+  }
+  pp_status st = read_ctl(c);
+  release(PP_OK);
+  if (st == PP_OK) st = check_device_error(c);
+  if (st != PP_OK) return st;
+  if (const unsigned why = c->h_ctl->stall) {
+    // given up: the input table is whole (its index may not be).  Next time
+    // with finer phases or more buckets, and after ever longer waits.
+    if (why & kPhaseClassFull) {
+      // a dense class of more active gates than its room (a star of bonds):
+      // then no phase has more gates than that
+      if (dense && c->phase_gates > kPhaseRank)
+        c->phase_gates = kPhaseRank;
+      else
+        c->phase_active = std::max(0.5, 0.6 * c->phase_active);
+    }
+    if (why & kPhaseBucketFull) {
+      c->phase_room = std::min(8.0, 2.0 * c->phase_room);
+      c->phase_active = std::max(0.5, 0.8 * c->phase_active);
+    }
+    if (why != kPhaseTableFull) c->phase_wait = std::min(32, (1 << std::min(c->phase_fails++, 5)) - 1);
+    return PP_OK;
+  }
+  c->phase_fails = 0;
+  if (c->cfg.profile_kernels) {
+    float ms = 0.f;
+    PP_CUDA(cudaEventElapsedTime(&ms, c->ev_layer[0], c->ev_layer[1]));
+    c->gate_ms += ms;
+    c->gates_timed++;
+  }
+  c->last_growth = (double)c->h_ctl->after_terms / (double)T;
+  if (want_activity) ent.activity.assign(c->h_activity, c->h_activity + G);
+  if (merge) {
+    PP_TRY(finish_queued_merge(c, src));
+  } else {
+    c->n_terms = c->h_ctl->n_terms;
+    c->n_live = c->h_ctl->n_live;
+    c->live_known = true;
+    PP_TRY(activate(c, dst));
+  }
+  *done = true;
+  return PP_OK;
 }
 
 // Everything pp_apply_layer does after the entry merge: damping, room, the
@@ -1214,8 +1472,17 @@ pp_status apply_layer_core(pp_ctx* c, std::vector<GateArgs>& args, const std::ve
     while ((double)grid_b * kBlock < (double)(est * rowf) * c->grid_scale) grid_b <<= 1;
     grid_b = std::min(grid_b, c->sms * (c->batched ? 8 : c->gate_bps));
   }
-  const GateArgs* d_args = nullptr;
-  if (layered && !args.empty()) PP_TRY(device_args(c, args, &d_args));
+  ArgsEntry* entry = nullptr;
+  if (layered && !args.empty()) PP_TRY(device_args(c, args, &entry));
+  const GateArgs* d_args = entry ? entry->d_args : nullptr;
+  if (entry && phases_allowed(c)) {
+    bool done = false;
+    PP_TRY(apply_layer_phased(c, *entry, args, symmetric_boundary && c->cfg.symmetry != PP_SYM_NONE,
+                              &done));
+    if (done) return PP_OK;
+  }
+  // the kernels below look partners up in the index in global memory
+  if (!c->index_ok && !args.empty()) PP_TRY(compact_into(c, 1 - c->active, 0.0, -1));
   // with a group (single column) the boundary merge is queued right behind the
   // gates, guarded by the stall flag, so one read of the control block serves both
   const bool queue_it = symmetric_boundary && c->cfg.symmetry != PP_SYM_NONE && !c->batched;
@@ -1239,7 +1506,7 @@ pp_status apply_layer_core(pp_ctx* c, std::vector<GateArgs>& args, const std::ve
       }
       PP_CUDA(launch_chain_finish(c->stream, c->d_ctl, (unsigned)args.size()));
       c->launches += 2;
-      if (queue_it) PP_TRY(queue_merge(c, c->cfg.symmetry));
+      if (queue_it) PP_TRY(queue_merge(c, c->cfg.symmetry, c->active, 1 - c->active));
       PP_TRY(read_ctl(c));
       PP_TRY(check_device_error(c));
       const unsigned end = c->h_ctl->stall ? c->h_ctl->stall - 1u : (unsigned)args.size();
@@ -1258,7 +1525,7 @@ pp_status apply_layer_core(pp_ctx* c, std::vector<GateArgs>& args, const std::ve
         const uint64_t after = c->h_ctl->after_terms;
         c->last_growth = (double)after / (double)n_start;
         if (queue_it) {
-          PP_TRY(finish_queued_merge(c));
+          PP_TRY(finish_queued_merge(c, 1 - c->active));
           merged_now = true;
         } else {
           c->n_terms = c->h_ctl->n_terms;
@@ -1368,6 +1635,7 @@ pp_status pp_destroy(pp_ctx* c) {
   if (c->stream) cudaStreamSynchronize(c->stream);
   pinned_put(c->h_ctl, sizeof(DevCtl));
   pinned_put(c->h_out, sizeof(double) * c->B);
+  pinned_put(c->h_activity, kActivityMax * sizeof(float));
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   delete c;
   return PP_OK;
@@ -1532,19 +1800,25 @@ pp_status pp_tune(pp_ctx* c, int n_gates, const pp_pauli* gates, const double* t
     double scale, factor;
     int persistent;
     int threads;  // block size of the persistent kernel
+    bool phased;  // layers as phases where they suit them
   };
   std::vector<Trial> trials;
   const int lk0 = c->cfg.layer_kernel ? 1 : 0;
+  const bool off0 = c->phase_off;
+  c->phase_off = false;
+  const bool can_phase = c->layer_bps > 0 && phases_allowed(c);
+  c->phase_off = off0;
+  if (can_phase) trials.push_back({c->grid_scale, 1.5, 1, kBlock, true});
   for (double f : {1.5, 3.0}) {
     if (c->batched) {
-      if (c->layer_bps > 0) trials.push_back({c->grid_scale, f, 1, kBlock});
+      if (c->layer_bps > 0) trials.push_back({c->grid_scale, f, 1, kBlock, false});
     } else {
       for (int k = 0; k < 2; ++k)
-        if (c->bps_by_threads[k] > 0) trials.push_back({c->grid_scale, f, 1, k ? 1024 : kBlock});
+        if (c->bps_by_threads[k] > 0) trials.push_back({c->grid_scale, f, 1, k ? 1024 : kBlock, false});
     }
-    trials.push_back({c->grid_scale, f, 0, c->layer_threads});
+    trials.push_back({c->grid_scale, f, 0, c->layer_threads, false});
   }
-  Trial best = {c->grid_scale, c->index_factor, lk0, c->layer_threads};
+  Trial best = {c->grid_scale, c->index_factor, lk0, c->layer_threads, can_phase && !off0};
   double best_ms = 1e300;
   auto run_trial = [&](const Trial& tr, pp_status* err) -> double {
     *err = PP_OK;
@@ -1555,6 +1829,7 @@ pp_status pp_tune(pp_ctx* c, int n_gates, const pp_pauli* gates, const double* t
       return 1e300;
     }
     c->cfg.layer_kernel = tr.persistent;
+    c->phase_off = !tr.phased;
     c->grid_scale = tr.scale;
     if (!c->batched) {
       c->layer_threads = tr.threads;
@@ -1576,6 +1851,7 @@ pp_status pp_tune(pp_ctx* c, int n_gates, const pp_pauli* gates, const double* t
   auto put_back = [&](const Trial& tr) {
     set_index_factor(c, tr.factor);
     c->cfg.layer_kernel = tr.persistent;
+    c->phase_off = !tr.phased;
     c->grid_scale = tr.scale;
     if (!c->batched) {
       c->layer_threads = tr.threads;
@@ -1596,6 +1872,7 @@ pp_status pp_tune(pp_ctx* c, int n_gates, const pp_pauli* gates, const double* t
     }
   }
   for (double scale : {0.5, 2.0, 4.0}) {
+    if (best.phased) break;  // phases size their own grid
     Trial tr = best;
     tr.scale = scale;
     pp_status st;
@@ -1998,4 +2275,11 @@ double ppk::layer_fraction_wanted(const pp_ctx* c) {
   if (!c || !c->cfg.layer_kernel || c->layer_bps <= 0) return 0.0;
   const double full = (double)c->sms * c->layer_bps;
   return std::min(1.0, (double)layer_grid_want(c, c->n_terms) / full);
+}
+
+size_t ppk::layer_scratch_bytes(const pp_ctx* c, int n_gates) {
+  if (!c || !c->cfg.layer_kernel || c->layer_bps <= 0 || !phases_allowed(c) || n_gates < kPhaseMinGates)
+    return 0;
+  const size_t bytes = phase_sizes(c, (size_t)n_gates, kPhaseMax).bytes;
+  return bytes > kPhaseBytesMax ? 0 : bytes;
 }

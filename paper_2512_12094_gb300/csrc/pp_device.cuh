@@ -244,8 +244,8 @@ __device__ __forceinline__ T warp_sum(T v) {
 
 // ----------------------------------------------------------- gate kernel
 
-template <int W>
-__device__ __forceinline__ int sigma_of(const GateArgs& g, const Key<W>& q) {
+template <int W, class Gate>
+__device__ __forceinline__ int sigma_of(const Gate& g, const Key<W>& q) {
   // P Q = i^E R with E = sum_sites px pz + qx qz + 2 pz qx - (px^qx)(pz^qz)
   // (P = i^{px pz} X^px Z^pz per site); i P Q = i^{E+1} R and E+1 is even.
   int e = g.pyy;

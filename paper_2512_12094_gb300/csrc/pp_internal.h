@@ -213,6 +213,84 @@ cudaError_t launch_sn_table(int n, cudaStream_t s, const double* bloch, double* 
 cudaError_t launch_pack_keys(int W, int n, int grid, cudaStream_t s, const uint64_t* x,
                              const uint64_t* z, uint64_t m, uint64_t* keys, unsigned* bad);
 
+// ------------------------------------------------------------- phases
+// A layer as a few phases over bucketed strings (pp_phase.cu, pp_phase.h).
+constexpr int kPhaseGates = 32;  // gates of a phase at most
+constexpr int kPhaseRank = 10;   // active gates of a dense class at most
+
+struct PhaseDesc {
+  int first, count, commuting;  // count 0: no phase (the dense table comes next)
+  int dense;                    // commuting, truncated, n <= 64: dense classes
+  unsigned skip;                // its gates that touch no string
+  int after, skip_after;        // gates of the layer behind it; those that touch no string
+  uint64_t ux[kMaxW], uz[kMaxW];
+};
+
+// [nb][cg] entries, cnt[nb] appended so far (may pass cg: the bucket was full).
+// meta: gates of the phase active on the string, low half of its class hash.
+struct PhaseBuckets {
+  uint32_t* keys;  // [2 P] words a string: x words, then z words
+  double* coef;
+  uint2* meta;
+  unsigned* cnt;
+};
+
+struct PhaseRule {
+  int use_eps;
+  uint64_t eps_bits;
+  int wmax;
+  const double* damp;  // per-gate noise, or nullptr
+};
+
+// Why a phased layer was given up (PhaseStat::fail).
+enum : unsigned {
+  kPhaseBucketFull = 1u,
+  kPhaseClassFull = 2u,  // one class outgrew a warp's shared memory
+  kPhaseTableFull = 4u,  // the destination table
+};
+
+struct alignas(16) PhaseStat {
+  unsigned fail, pad;
+  unsigned long long live0;  // live strings entering the first gate
+  // of the dense phases: change of the sum of live strings entering the gates
+  // behind, of the same over gates that touch nothing, anticommuting strings
+  long long upd, skipped;
+  unsigned long long ac, pad2;
+};
+
+// Accumulators of a phased layer; all but activity start at zero.
+struct PhaseAcc {
+  PhaseStat* st;
+  long long* delta;        // [gates] change of the live count
+  unsigned long long* ac;  // [gates] live anticommuting strings
+  unsigned* touch;         // [gates] some string may anticommute (or be damped)
+  unsigned* seen;          // [gates] of dense phases: strings of the counted buckets active in it
+  float* activity;         // [gates] ac / live, written by launch_phase_end
+};
+
+// 32-bit words per plane that phases keep a string of n qubits in (P below),
+// the warps of a phase kernel an SM holds, and the strings one of them holds.
+int phase_words(int n);
+int phase_warps_per_sm();
+int phase_strings_per_warp(int P);
+// Zero clear_bytes from acc.st on and reset the context's append cursor,
+// occupancy masks and stall flag.
+cudaError_t launch_phase_begin(cudaStream_t s, const PhaseAcc& acc, size_t clear_bytes, DevCtl* ctl,
+                               int sms);
+// Live entries of src[0, T) into the buckets of phase d.
+cudaError_t launch_phase_deal(int P, int grid, cudaStream_t s, const DevTable& src, uint64_t T,
+                              int use_eps, const PhaseBuckets& out, unsigned nb, unsigned cg,
+                              const PhaseDesc& d, const GateArgs* gates, const PhaseAcc& acc);
+// Phase d from `in`, on `warps` warps; survivors into `out` (the buckets of `next`) or, when
+// next.count is 0, appended to dense at ctl->n_next.
+cudaError_t launch_phase(int P, int warps, cudaStream_t s, const PhaseBuckets& in,
+                         const PhaseBuckets& out, unsigned nb, unsigned cg, const PhaseDesc& d,
+                         const PhaseDesc& next, const GateArgs* gates, const PhaseRule& rule,
+                         const DevTable& dense, DevCtl* ctl, const PhaseAcc& acc);
+// Statistics and table size into ctl; a failed layer sets ctl->stall to the
+// fail bits instead.
+cudaError_t launch_phase_end(cudaStream_t s, DevCtl* ctl, const PhaseAcc& acc, unsigned n_gates);
+
 // Message returned by pp_last_error() on the calling thread.
 void set_last_error(const std::string& msg);
 
@@ -230,6 +308,9 @@ void set_grid_fraction(pp_ctx* c, double frac);
 // The fraction of the GPU's co-resident blocks the context's next persistent
 // layer launch would use with no limit (0 when it has no persistent path).
 double layer_fraction_wanted(const pp_ctx* c);
+// Device memory beyond what it holds that the context's next layer of n_gates
+// gates could use while it runs (0: none; it does without where there is none).
+size_t layer_scratch_bytes(const pp_ctx* c, int n_gates);
 
 // ------------------------------------------------------- batched launchers
 // Same contracts as the single-column kernels above, on B-column rows.

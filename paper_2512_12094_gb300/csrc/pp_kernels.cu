@@ -445,6 +445,7 @@ struct LayerSmem {
   GateShared<NT> sh;
   GateArgs gate[2];  // current gate and the prefetched next one
   int ok;
+  unsigned skip;     // first gate of a round that touches a string
 };
 
 // Blocks of NT threads: 256 (four or two per SM) or 1024 (one per SM: a
@@ -498,13 +499,40 @@ __global__ void __launch_bounds__(NT, NT == 1024 ? 1 : ((W == 1) ? 4 : 2))
       if (g.damp) touch |= g.supp[j] & (ox[j] | oz[j]);
     }
     if (touch == 0) {
-      if (blockIdx.x == 0 && threadIdx.x == 0) {
-        atomicAdd(&ctl->updates, (double)L0);
-        atomicAdd(&ctl->gates_done, 1ull);
-        atomicAdd(&ctl->skipped_updates, (double)L0);
-        atomicAdd(&ctl->gates_skipped, 1ull);
+      // a run of such gates: every thread tests one of the gates that follow
+      // (a layer of 6048 gates over strings on a few qubits skips all but some
+      // 400 of them; one after the other they took 0.45 us each)
+      unsigned nxt = gid + 1;
+      while (nxt < n_gates) {
+        __syncthreads();  // the last round's readers of S.skip are done
+        if (threadIdx.x == 0) S.skip = NT;
+        __syncthreads();
+        const unsigned k = nxt + threadIdx.x;
+        uint64_t t = 0;
+        if (k < n_gates) {
+#pragma unroll
+          for (int j = 0; j < W; ++j) {
+            const uint64_t px = __ldg(&gates[k].px[j]), pz = __ldg(&gates[k].pz[j]);
+            t |= (px & oz[j]) | (pz & ox[j]);
+            if (g.damp) t |= (px | pz) & (ox[j] | oz[j]);
+          }
+        }
+        const unsigned bal = __ballot_sync(kFull, t != 0);
+        if (bal && (threadIdx.x & 31) == 0) atomicMin(&S.skip, threadIdx.x + __ffs(bal) - 1);
+        __syncthreads();
+        const unsigned f = S.skip;
+        nxt = min(nxt + f, n_gates);
+        if (f < NT) break;
       }
-      if (gid + 1 < n_gates) fetch_args(gid + 1, buf ^ 1);
+      if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const unsigned run = nxt - gid;
+        atomicAdd(&ctl->updates, (double)L0 * run);
+        atomicAdd(&ctl->gates_done, (unsigned long long)run);
+        atomicAdd(&ctl->skipped_updates, (double)L0 * run);
+        atomicAdd(&ctl->gates_skipped, (unsigned long long)run);
+      }
+      if (nxt < n_gates) fetch_args(nxt, buf ^ 1);
+      gid = nxt - 1;
       continue;
     }
     if (!gate_fits(t, T0)) {  // the same decision in every block
