@@ -209,6 +209,17 @@ Grow grow_reservation(pp_server* s, Job& j, size_t want) {
   }
 }
 
+// Raise a running job's reservation to `want` if the memory is free at once (for
+// what a layer can do without).
+bool try_grow_reservation(pp_server* s, Job& j, size_t want) {
+  std::lock_guard<std::mutex> lock(s->mu);
+  if (want <= j.reserve || s->growing > 0 || s->reserved - j.reserve + want > s->budget) return false;
+  s->reserved += want - j.reserve;
+  j.reserve = want;
+  j.grows++;
+  return true;
+}
+
 // Run one job on `stream`: returns its status; fills r.  *give_back is set
 // when the job released its memory to let others finish (it is queued
 // again).
@@ -262,6 +273,11 @@ pp_status run_job(pp_server* s, Job& j, cudaStream_t stream, pp_job_result& r, b
           break;
         }
       }
+      // scratch with which the layer runs as phases, several times faster; the
+      // copy of the table that a budgeted layer keeps comes on top of it
+      const size_t scratch = ppk::layer_scratch_bytes(ctx, (int)j.gates.size());
+      if (scratch && try_grow_reservation(s, j, round_mib((double)(2 * stats.device_bytes + scratch))))
+        pp_set_budget(ctx, j.reserve);
     }
     for (;;) {
       // A layer runs in one persistent launch on the share units it holds
