@@ -1203,11 +1203,21 @@ uint64_t layer_grid_want(const pp_ctx* c, uint64_t n_now) {
   return std::min<uint64_t>(std::max<uint64_t>(want, 1), full);
 }
 
-// Phases take the place of the persistent layer kernel on single FP64 columns.
+// Dense classes (pp_phase.cu): one or two words, no damping per gate (which changes
+// strings that a gate commutes with), truncation on -- rows need none, as which
+// of them live is kept apart.
+bool dense_classes(const pp_ctx* c) {
+  return c->n <= 64 && (c->batched || c->cfg.coeff_eps > 0.0) &&
+         c->cfg.noise_mode != PP_NOISE_PER_GATE;
+}
+
+// Phases take the place of the persistent layer kernel, on rows where all of them
+// have dense classes.
 // A caller that sets the block size of that kernel, or the limit of the waits
 // at its barriers, asks for it; pp_tune may have measured it faster.
 bool phases_allowed(const pp_ctx* c) {
-  return !c->batched && c->cfg.block_threads == 0 && c->cfg.wait_limit == 0 && !c->phase_off;
+  return (!c->batched || dense_classes(c)) && c->cfg.block_threads == 0 && c->cfg.wait_limit == 0 &&
+         !c->phase_off;
 }
 
 // Apply the layer as phases (pp_phase.cu) and, with merge, its symmetry merge.
@@ -1219,18 +1229,13 @@ bool phases_allowed(const pp_ctx* c) {
 // pass per gate costs one and a barrier.
 constexpr int kPhaseMinGates = 3;
 constexpr int kPhaseMax = 64;       // phases of a layer
+constexpr double kRowsFill = 8.0;    // of rows
 constexpr double kDenseFill = 700.0; // strings of a bucket in the expected table, dense classes
 constexpr int kPhaseBits = 10;      // key bits a run that does not commute may touch
 
 constexpr size_t kPhaseBytesMax = (size_t)64 << 30;
 
 size_t align256(size_t b) { return (b + 255) / 256 * 256; }
-
-// Dense classes (pp_phase.cu): one or two words, truncation on, no damping per
-// gate (which changes strings that a gate commutes with).
-bool dense_classes(const pp_ctx* c) {
-  return c->n <= 64 && c->cfg.coeff_eps > 0.0 && c->cfg.noise_mode != PP_NOISE_PER_GATE;
-}
 
 // Buckets of a phased layer of G gates in P phases, and its scratch.  One bucket
 // per resident warp (dense: block) at least, and enough that a bucket of the
@@ -1240,7 +1245,7 @@ bool dense_classes(const pp_ctx* c) {
 struct PhaseSizes {
   double est;  // strings expected at the layer's end
   uint64_t nb, cg;
-  size_t clear, bytes;
+  size_t clear, bytes, rows = 0, spill = 0;
 };
 
 PhaseSizes phase_sizes(const pp_ctx* c, size_t G, size_t P) {
@@ -1248,13 +1253,22 @@ PhaseSizes phase_sizes(const pp_ctx* c, size_t G, size_t P) {
   const int P32 = phase_words(c->n);
   const bool dense = dense_classes(c);
   z.est = (double)c->n_terms * std::max(1.5, 1.25 * c->last_growth);
-  const double half = dense ? kDenseFill : 0.5 * phase_strings_per_warp(P32);
-  const uint64_t least = (uint64_t)c->sms * (dense ? 2 : phase_warps_per_sm());
+  const double half = c->batched ? kRowsFill
+                      : dense    ? kDenseFill
+                                 : 0.5 * phase_strings_per_warp(P32);
+  const uint64_t least = (uint64_t)c->sms * (c->batched ? 8 : dense ? 2 : phase_warps_per_sm());
   z.nb = std::max<uint64_t>(least, (uint64_t)std::ceil(z.est * c->phase_room / half));
   z.cg = (256 + (uint64_t)(4.0 * z.est / (double)z.nb)) / 8 * 8;
-  z.clear = sizeof(PhaseStat) + G * 24 + P * z.nb * 4;
+  z.clear = sizeof(PhaseStat) + G * 24 + P * 8 + P * z.nb * 4;
   z.bytes = align256(z.clear) + align256(G * 4) +
             2 * (align256(z.nb * z.cg * 8 * P32) + 2 * align256(z.nb * z.cg * 8));
+  if (c->batched) {
+    // rows of the phases between, and of classes larger than shared memory
+    const size_t row = (size_t)c->B * c->esize;
+    z.rows = P >= 2 ? align256(c->buf[c->active].cap * row) : 0;
+    z.spill = align256(rows_launch(P32, c->B, (int)c->esize, c->sms, c->grid_frac).spill_rows * row);
+    z.bytes += z.rows + z.spill;
+  }
   return z;
 }
 
@@ -1289,6 +1303,9 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
       ppphase::plan(gens, c->W, touch.data(), ent.activity.data(), lim);
   const size_t P = phases.size();
   if (P == 0 || P > (size_t)kPhaseMax || P * kPhaseMinGates > n_touch) return PP_OK;
+  if (c->batched)
+    for (const ppphase::Phase& ph : phases)
+      if (!ph.triangular) return PP_OK;
   Range range_("phases");
   const PhaseSizes z = phase_sizes(c, G, P);
   const uint64_t nb = z.nb, cg = z.cg;
@@ -1315,9 +1332,11 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   acc.ac = reinterpret_cast<unsigned long long*>(acc.delta + G);
   acc.touch = reinterpret_cast<unsigned*>(acc.ac + G);
   acc.seen = acc.touch + G;
-  unsigned* cnt = acc.seen + G;
+  unsigned long long* written = reinterpret_cast<unsigned long long*>(acc.seen + G);  // rows per phase
+  unsigned* cnt = reinterpret_cast<unsigned*>(written + P);
   acc.activity = reinterpret_cast<float*>(scratch + al(clear));
   PhaseBuckets buckets[2];
+  unsigned char *mid_rows, *spill;
   {
     unsigned char* p = scratch + al(clear) + al(G * 4);
     for (int k = 0; k < 2; ++k) {
@@ -1329,6 +1348,8 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
       p += al(nb * cg * 8);
       buckets[k].cnt = nullptr;
     }
+    mid_rows = p;
+    spill = p + z.rows;
   }
   std::vector<int> skip_after(G + 1, 0);  // gates from g on that touch nothing
   for (size_t g = G; g-- > 0;) skip_after[g] = skip_after[g + 1] + !touch[g];
@@ -1351,6 +1372,7 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   };
   PhaseRule rule;
   rule.use_eps = args[0].use_eps;
+  rule.eps = args[0].eps;
   rule.eps_bits = args[0].eps_bits;
   rule.wmax = args[0].wmax;
   rule.damp = args[0].damp;
@@ -1361,14 +1383,34 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   run(launch_phase_begin(c->stream, acc, clear, c->d_ctl, c->sms));
   buckets[0].cnt = cnt;
   const int dgrid = (int)std::min<uint64_t>((T + kBlock - 1) / kBlock, (uint64_t)c->sms * 8);
-  run(launch_phase_deal(P32, dgrid, c->stream, desc_of(c, c->buf[src]), T, rule.use_eps, buckets[0],
-                        (unsigned)nb, (unsigned)cg, desc(0), ent.d_args, acc));
-  for (size_t p = 0; p < P; ++p) {
-    PhaseBuckets in = buckets[p & 1], out = buckets[(p + 1) & 1];
-    in.cnt = cnt + p * nb;
-    out.cnt = p + 1 < P ? cnt + (p + 1) * nb : nullptr;
-    run(launch_phase(P32, warps, c->stream, in, out, (unsigned)nb, (unsigned)cg, desc(p), desc(p + 1),
-                     ent.d_args, rule, desc_of(c, c->buf[dst]), c->d_ctl, acc));
+  if (c->batched) {
+    const RowsLaunch L = rows_launch(P32, c->B, (int)c->esize, c->sms, c->grid_frac);
+    run(launch_rows_deal(P32, dgrid, c->stream, desc_of(c, c->buf[src]), T, buckets[0], (unsigned)nb,
+                         (unsigned)cg, desc(0), ent.d_args, acc));
+    const void* from = c->buf[src].rows;
+    for (size_t p = 0; p < P; ++p) {
+      PhaseBuckets in = buckets[p & 1], out = buckets[(p + 1) & 1];
+      in.cnt = cnt + p * nb;
+      out.cnt = p + 1 < P ? cnt + (p + 1) * nb : nullptr;
+      // the last phase writes the destination table's rows, those before it
+      // take turns with the rows between; the source's stay whole
+      void* to = (P - 1 - p) % 2 == 0 ? c->buf[dst].rows : (void*)mid_rows;
+      run(launch_rows_phase(P32, L, c->stream, in, out, (unsigned)nb, (unsigned)cg, desc(p), desc(p + 1),
+                            ent.d_args, rule, from, to, c->buf[dst].cap,
+                            p + 1 < P ? written + p : &c->d_ctl->n_next, spill,
+                            desc_of(c, c->buf[dst]), c->d_ctl, acc));
+      from = to;
+    }
+  } else {
+    run(launch_phase_deal(P32, dgrid, c->stream, desc_of(c, c->buf[src]), T, rule.use_eps, buckets[0],
+                          (unsigned)nb, (unsigned)cg, desc(0), ent.d_args, acc));
+    for (size_t p = 0; p < P; ++p) {
+      PhaseBuckets in = buckets[p & 1], out = buckets[(p + 1) & 1];
+      in.cnt = cnt + p * nb;
+      out.cnt = p + 1 < P ? cnt + (p + 1) * nb : nullptr;
+      run(launch_phase(P32, warps, c->stream, in, out, (unsigned)nb, (unsigned)cg, desc(p), desc(p + 1),
+                       ent.d_args, rule, desc_of(c, c->buf[dst]), c->d_ctl, acc));
+    }
   }
   run(launch_phase_end(c->stream, c->d_ctl, acc, (unsigned)G));
   if (c->cfg.profile_kernels) run(cudaEventRecord(c->ev_layer[1], c->stream));
@@ -1477,9 +1519,9 @@ pp_status apply_layer_core(pp_ctx* c, std::vector<GateArgs>& args, const std::ve
   const GateArgs* d_args = entry ? entry->d_args : nullptr;
   if (entry && phases_allowed(c)) {
     bool done = false;
-    PP_TRY(apply_layer_phased(c, *entry, args, symmetric_boundary && c->cfg.symmetry != PP_SYM_NONE,
-                              &done));
-    if (done) return PP_OK;
+    const bool merge = symmetric_boundary && c->cfg.symmetry != PP_SYM_NONE;
+    PP_TRY(apply_layer_phased(c, *entry, args, merge && !c->batched, &done));
+    if (done) return merge && c->batched ? merge_active(c, c->cfg.symmetry) : PP_OK;
   }
   // the kernels below look partners up in the index in global memory
   if (!c->index_ok && !args.empty()) PP_TRY(compact_into(c, 1 - c->active, 0.0, -1));
@@ -2278,7 +2320,8 @@ double ppk::layer_fraction_wanted(const pp_ctx* c) {
 }
 
 size_t ppk::layer_scratch_bytes(const pp_ctx* c, int n_gates) {
-  if (!c || !c->cfg.layer_kernel || c->layer_bps <= 0 || !phases_allowed(c) || n_gates < kPhaseMinGates)
+  if (!c || c->batched || !c->cfg.layer_kernel || c->layer_bps <= 0 || !phases_allowed(c) ||
+      n_gates < kPhaseMinGates)
     return 0;
   const size_t bytes = phase_sizes(c, (size_t)n_gates, kPhaseMax).bytes;
   return bytes > kPhaseBytesMax ? 0 : bytes;

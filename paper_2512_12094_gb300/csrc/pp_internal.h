@@ -237,6 +237,7 @@ struct PhaseBuckets {
 
 struct PhaseRule {
   int use_eps;
+  double eps;
   uint64_t eps_bits;
   int wmax;
   const double* damp;  // per-gate noise, or nullptr
@@ -287,6 +288,24 @@ cudaError_t launch_phase(int P, int warps, cudaStream_t s, const PhaseBuckets& i
                          const PhaseBuckets& out, unsigned nb, unsigned cg, const PhaseDesc& d,
                          const PhaseDesc& next, const GateArgs* gates, const PhaseRule& rule,
                          const DevTable& dense, DevCtl* ctl, const PhaseAcc& acc);
+// Batched layers (pp_phase_rows.cu; n <= 64, dense phases only): buckets hold row
+// numbers in place of coefficients.
+struct RowsLaunch {
+  int threads, grid, smem_rows;  // rows of a class held in shared memory
+  size_t smem, spill_rows;       // rows of scratch in global memory for larger classes
+};
+RowsLaunch rows_launch(int P, int B, int esize, int sms, double fraction);
+cudaError_t launch_rows_deal(int P, int grid, cudaStream_t s, const DevTable& src, uint64_t T,
+                             const PhaseBuckets& out, unsigned nb, unsigned cg, const PhaseDesc& d,
+                             const GateArgs* gates, const PhaseAcc& acc);
+// Phase d: rows src -> dst (room for dst_cap, *n_out written so far); after the
+// last phase keys and liveness of `dense` too, whose B and f32 describe the rows.
+cudaError_t launch_rows_phase(int P, const RowsLaunch& L, cudaStream_t s, const PhaseBuckets& in,
+                              const PhaseBuckets& out, unsigned nb, unsigned cg, const PhaseDesc& d,
+                              const PhaseDesc& next, const GateArgs* gates, const PhaseRule& rule,
+                              const void* src, void* dst, uint64_t dst_cap, unsigned long long* n_out,
+                              void* spill, const DevTable& dense, DevCtl* ctl, const PhaseAcc& acc);
+
 // Statistics and table size into ctl; a failed layer sets ctl->stall to the
 // fail bits instead.
 cudaError_t launch_phase_end(cudaStream_t s, DevCtl* ctl, const PhaseAcc& acc, unsigned n_gates);

@@ -142,3 +142,48 @@ def test_phases_with_a_memory_budget():
     for t in tables[1:]:
         for u, v in zip(tables[0], t):
             np.testing.assert_array_equal(u, v)
+
+
+def batched_pair(n, B, f32, eps, wmax, layers, group=0):
+    angles = pi.batched_ring_angles(B, n)
+    gx, gz, _ = pi.Circuit(n, [pi.ring_layer(n, 0.0, 0.0, 0.0)]).gate_arrays(0)
+    th = np.repeat(angles.T, n, axis=0)
+    th = th[:, 0].copy() if B == 1 else th
+    x, z, c = pi.mean_z(n).arrays()
+    coef = np.repeat(c[:, None], B, axis=1)
+    kw = dict(symmetry=group, eps=eps, max_weight=wmax, batch=B, f32=f32)
+    a = pp.Propagator(n, x, z, coef, **kw)
+    b = pp.Propagator(n, x, z, coef, block_threads=256, **kw)
+    for _ in range(layers):
+        a.apply_layer(gx, gz, th, True)
+        b.apply_layer(gx, gz, th, True)
+        assert a.num_terms()[0] == b.num_terms()[0]
+    sa, sb = a.stats(), b.stats()
+    for k in KEYS:
+        assert sa[k] == sb[k], k
+    ta, tb = sorted_table(a), sorted_table(b)
+    np.testing.assert_array_equal(ta[0], tb[0])
+    np.testing.assert_array_equal(ta[1], tb[1])
+    if group == 0:
+        np.testing.assert_array_equal(ta[2], tb[2])
+    else:
+        np.testing.assert_allclose(ta[2], tb[2], rtol=0, atol=1e-6 if f32 else 1e-12)
+    a.close()
+    b.close()
+    return len(ta[0])
+
+
+@pytest.mark.parametrize("n,B,f32,eps,wmax,layers", [
+    (1, 4, False, 0.0, -1, 2), (5, 3, False, 0.0, -1, 3), (9, 1, True, 1e-4, -1, 4),
+    (16, 31, True, 1e-4, 6, 3), (32, 33, False, 1e-5, -1, 3), (33, 256, False, 1e-5, -1, 2),
+    (64, 256, True, 1e-5, -1, 3), (40, 300, False, 1e-4, 5, 2), (12, 512, False, 1e-6, -1, 3),
+    (11, 64, False, 0.0, -1, 4)])
+def test_rows_bit_for_bit(n, B, f32, eps, wmax, layers):
+    """Rows at column counts below, at and above a block, both types, classes
+    that fit shared memory and classes that do not."""
+    batched_pair(n, B, f32, eps, wmax, layers)
+
+
+@pytest.mark.parametrize("f32", [False, True])
+def test_rows_merged(f32):
+    assert batched_pair(14, 20, f32, 1e-4, -1, 3, group=1) > 100
