@@ -643,7 +643,6 @@ using ppsym::bloch_invariant;
 using ppsym::generators;
 using ppsym::group_kind;
 using ppsym::group_lx;
-using ppsym::HKey;
 using ppsym::multiset_invariant;
 using ppsym::valid_group;
 
@@ -708,23 +707,25 @@ pp_status ingest_terms(pp_ctx* c, int64_t n_terms, const uint64_t* x, const uint
   } else if (c->cfg.symmetry != PP_SYM_NONE) {
     // the observable is invariant when every column is
     c->obs_invariant = true;
+    const int K = 2 * W;
+    std::vector<uint64_t> keys((size_t)n_terms * K), uniq;
+    for (int64_t i = 0; i < n_terms; ++i)
+      for (int j = 0; j < W; ++j) {
+        keys[(size_t)i * K + j] = hx[i * W + j];
+        keys[(size_t)i * K + W + j] = hz[i * W + j];
+      }
+    // equal strings accumulate, in the order they came
+    const std::vector<uint32_t> at = ppsym::key_order(keys.data(), (size_t)n_terms, K);
+    std::vector<uint32_t> group_of((size_t)n_terms);
+    for (size_t i = 0; i < at.size(); ++i) {
+      const uint64_t* k = &keys[(size_t)at[i] * K];
+      if (i == 0 || !std::equal(k, k + K, uniq.end() - K)) uniq.insert(uniq.end(), k, k + K);
+      group_of[i] = (uint32_t)(uniq.size() / K - 1);
+    }
     for (int b = 0; b < c->B && c->obs_invariant; ++b) {
-      std::map<HKey, double> acc;
-      for (int64_t i = 0; i < n_terms; ++i) {
-        HKey k(2 * W);
-        for (int j = 0; j < W; ++j) {
-          k[j] = hx[i * W + j];
-          k[W + j] = hz[i * W + j];
-        }
-        acc[k] += hc[(size_t)i * c->B + b];
-      }
-      std::vector<HKey> ks;
-      std::vector<double> vs;
-      for (auto& kv : acc) {
-        ks.push_back(kv.first);
-        vs.push_back(kv.second);
-      }
-      c->obs_invariant = multiset_invariant(c->cfg.symmetry, c->n, W, ks, vs, 1e-12);
+      std::vector<double> vs(uniq.size() / K, 0.0);
+      for (size_t i = 0; i < at.size(); ++i) vs[group_of[i]] += hc[(size_t)at[i] * c->B + b];
+      c->obs_invariant = multiset_invariant(c->cfg.symmetry, c->n, W, uniq.data(), vs.data(), vs.size(), 1e-12);
     }
   }
 
@@ -942,18 +943,21 @@ pp_status build_gates(pp_ctx* c, int n_gates, const pp_pauli* gates, const doubl
   return PP_OK;
 }
 
-// Device copy of a byte block, cached by content (gate arguments, per-gate
-// cos/sin columns).
-pp_status cached_upload(pp_ctx* c, std::vector<ArgsEntry>& cache,
-                        std::vector<unsigned char>&& bytes, const void** out) {
+// The device block cached under `key` (by content), or nullptr.
+const void* cached_block(pp_ctx* c, std::vector<ArgsEntry>& cache, const std::vector<unsigned char>& key) {
   c->graph_clock++;
   for (auto& e : cache) {
-    if (e.sig == bytes) {
+    if (e.sig == key) {
       e.last_use = c->graph_clock;
-      *out = e.d_args;
-      return PP_OK;
+      return e.d_args;
     }
   }
+  return nullptr;
+}
+
+// Device copy of a byte block, kept under `key` (the 16 used last are kept).
+pp_status cached_upload(pp_ctx* c, std::vector<ArgsEntry>& cache, std::vector<unsigned char>&& key,
+                        const std::vector<unsigned char>& bytes, const void** out) {
   if (cache.size() >= 16) {
     auto it = std::min_element(cache.begin(), cache.end(), [](const ArgsEntry& a, const ArgsEntry& b) {
       return a.last_use < b.last_use;
@@ -965,7 +969,7 @@ pp_status cached_upload(pp_ctx* c, std::vector<ArgsEntry>& cache,
   ent.n = bytes.size();
   PP_TRY(dmalloc(c, (void**)&ent.d_args, ent.n));
   PP_CUDA(upload(c, ent.d_args, bytes.data(), ent.n));
-  ent.sig = std::move(bytes);
+  ent.sig = std::move(key);
   ent.last_use = c->graph_clock;
   *out = ent.d_args;
   cache.push_back(std::move(ent));
@@ -977,24 +981,31 @@ pp_status cached_upload(pp_ctx* c, std::vector<ArgsEntry>& cache,
 pp_status batched_columns(pp_ctx* c, std::vector<GateArgs>& args, const std::vector<int>& src,
                           const double* theta) {
   const int B = c->B;
-  std::vector<unsigned char> bytes(args.size() * 2 * B * c->esize);
-  for (size_t k = 0; k < args.size(); ++k) {
-    const double* th = theta + (size_t)src[k] * B;
-    for (int b = 0; b < B; ++b) {
-      const double cv = std::cos(th[b]), sv = std::sin(th[b]);
-      if (c->f32) {
-        float* f = reinterpret_cast<float*>(bytes.data()) + k * 2 * B;
-        f[b] = (float)cv;
-        f[B + b] = (float)sv;
-      } else {
-        double* d = reinterpret_cast<double*>(bytes.data()) + k * 2 * B;
-        d[b] = cv;
-        d[B + b] = sv;
+  // found by the angles: their cosines and sines are taken once per layer that
+  // repeats, not once per call (192 gates x 256 columns: 1 ms)
+  std::vector<unsigned char> angles(args.size() * B * sizeof(double));
+  for (size_t k = 0; k < args.size(); ++k)
+    memcpy(angles.data() + k * B * sizeof(double), theta + (size_t)src[k] * B, B * sizeof(double));
+  const void* dev = nullptr;
+  if (!(dev = cached_block(c, c->cs_cache, angles))) {
+    std::vector<unsigned char> bytes(args.size() * 2 * B * c->esize);
+    for (size_t k = 0; k < args.size(); ++k) {
+      const double* th = theta + (size_t)src[k] * B;
+      for (int b = 0; b < B; ++b) {
+        const double cv = std::cos(th[b]), sv = std::sin(th[b]);
+        if (c->f32) {
+          float* f = reinterpret_cast<float*>(bytes.data()) + k * 2 * B;
+          f[b] = (float)cv;
+          f[B + b] = (float)sv;
+        } else {
+          double* d = reinterpret_cast<double*>(bytes.data()) + k * 2 * B;
+          d[b] = cv;
+          d[B + b] = sv;
+        }
       }
     }
+    PP_TRY(cached_upload(c, c->cs_cache, std::move(angles), bytes, &dev));
   }
-  const void* dev = nullptr;
-  PP_TRY(cached_upload(c, c->cs_cache, std::move(bytes), &dev));
   for (size_t k = 0; k < args.size(); ++k)
     args[k].csb = static_cast<const unsigned char*>(dev) + k * 2 * B * c->esize;
   return PP_OK;
@@ -1704,19 +1715,17 @@ pp_status pp_apply_layer(pp_ctx* c, int n_gates, const pp_pauli* gates, const do
     for (const auto& v : c->sym_ok) validated |= (v == sig);
   }
   if (c->cfg.symmetry != PP_SYM_NONE && c->cfg.check_symmetry && n_gates > 0 && !validated) {
-    std::vector<HKey> ks;
-    for (int t = 0; t < n_gates; ++t) {
-      HKey k(2 * c->W);
+    const int K = 2 * c->W;
+    std::vector<uint64_t> ks((size_t)n_gates * K);
+    for (int t = 0; t < n_gates; ++t)
       for (int j = 0; j < c->W; ++j) {
-        k[j] = gates[t].x[j];
-        k[c->W + j] = gates[t].z[j];
+        ks[(size_t)t * K + j] = gates[t].x[j];
+        ks[(size_t)t * K + c->W + j] = gates[t].z[j];
       }
-      ks.push_back(k);
-    }
     for (int b = 0; b < c->B; ++b) {
       std::vector<double> vs(n_gates);
       for (int t = 0; t < n_gates; ++t) vs[t] = theta[(size_t)t * c->B + b];
-      if (!multiset_invariant(c->cfg.symmetry, c->n, c->W, ks, vs, 0.0))
+      if (!multiset_invariant(c->cfg.symmetry, c->n, c->W, ks.data(), vs.data(), vs.size(), 0.0))
         return fail(PP_ERR_SYMMETRY, "layer gate multiset is not invariant under the group");
     }
     if (c->sym_ok.size() >= 8) c->sym_ok.erase(c->sym_ok.begin());
@@ -2002,8 +2011,11 @@ pp_status pp_expect(pp_ctx* c, const double* bloch, double* out) {
     for (int q = 0; q < n; ++q)
       if (bloch[3 * q + 2] == -1.0) a.bits[q >> 6] |= 1ull << (q & 63);
   }
-  PP_CUDA(cudaMemcpyAsync(c->d_bloch, bloch, sizeof(double) * 3 * n, cudaMemcpyHostToDevice,
-                          c->stream));
+  // a basis state travels in the arguments, except to the kernels that take it as
+  // a product state
+  if (!a.basis || (a.group != PP_SYM_NONE && a.group != PP_SYM_ZN))
+    PP_CUDA(cudaMemcpyAsync(c->d_bloch, bloch, sizeof(double) * 3 * n, cudaMemcpyHostToDevice,
+                            c->stream));
   a.bloch = c->d_bloch;
   if (a.group == PP_SYM_SN) {
     size_t sn = (size_t)(n + 1) * (n + 1) * (n + 1);

@@ -9,26 +9,22 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
-#include <map>
 #include <vector>
 
 #include "../../include/pp.h"
 
 namespace ppsym {
 
-inline void get_bit(const uint64_t* m, int q, int& b) { b = (int)((m[q >> 6] >> (q & 63)) & 1ull); }
-
 inline void permute_string(const uint64_t* x, const uint64_t* z, int n, int W,
                            const std::vector<int>& to, uint64_t* ox, uint64_t* oz) {
+  (void)n;
   for (int j = 0; j < W; ++j) ox[j] = oz[j] = 0;
-  for (int q = 0; q < n; ++q) {
-    int xb, zb;
-    get_bit(x, q, xb);
-    get_bit(z, q, zb);
-    int t = to[q];
-    ox[t >> 6] |= (uint64_t)xb << (t & 63);
-    oz[t >> 6] |= (uint64_t)zb << (t & 63);
-  }
+  for (int j = 0; j < W; ++j)  // the sites that hold a letter
+    for (uint64_t m = x[j] | z[j]; m; m &= m - 1) {
+      const int b = __builtin_ctzll(m), t = to[64 * j + b];
+      ox[t >> 6] |= ((x[j] >> b) & 1ull) << (t & 63);
+      oz[t >> 6] |= ((z[j] >> b) & 1ull) << (t & 63);
+    }
 }
 
 // Group codes: kind in the low byte (pp_symmetry), torus width above it.
@@ -78,32 +74,71 @@ inline std::vector<std::vector<int>> generators(int group, int n) {
 
 typedef std::vector<uint64_t> HKey;
 
+// Positions of m keys of K words each in ascending order, equal keys in the
+// order they came.
+inline std::vector<uint32_t> key_order(const uint64_t* keys, size_t m, int K) {
+  std::vector<uint32_t> at(m);
+  for (size_t i = 0; i < m; ++i) at[i] = (uint32_t)i;
+  std::sort(at.begin(), at.end(), [&](uint32_t a, uint32_t b) {
+    const uint64_t *p = keys + (size_t)a * K, *q = keys + (size_t)b * K;
+    for (int j = 0; j < K; ++j)
+      if (p[j] != q[j]) return p[j] < q[j];
+    return a < b;
+  });
+  return at;
+}
+
 // Is the multiset {(string_i, value_i)} mapped onto itself by every generator?
-inline bool multiset_invariant(int group, int n, int W, const std::vector<HKey>& keys,
-                               const std::vector<double>& vals, double rel_tol) {
-  std::map<HKey, std::vector<double>> base;
-  for (size_t i = 0; i < keys.size(); ++i) base[keys[i]].push_back(vals[i]);
-  for (auto& kv : base) std::sort(kv.second.begin(), kv.second.end());
-  for (const auto& g : generators(group, n)) {
-    std::map<HKey, std::vector<double>> img;
-    for (size_t i = 0; i < keys.size(); ++i) {
-      HKey k(2 * W);
-      permute_string(keys[i].data(), keys[i].data() + W, n, W, g, k.data(), k.data() + W);
-      img[k].push_back(vals[i]);
+// keys: m strings, x words then z words.  Both sides are sorted by string and,
+// within equal strings, by value, and compared place by place (a map of vectors
+// took 1 us a string and generator).
+inline bool multiset_invariant(int group, int n, int W, const uint64_t* keys, const double* vals,
+                               size_t m, double rel_tol) {
+  const int K = 2 * W;
+  auto equal = [&](const uint64_t* p, const uint64_t* q) {
+    for (int j = 0; j < K; ++j)
+      if (p[j] != q[j]) return false;
+    return true;
+  };
+  // values in the order of at, sorted within equal keys
+  auto sorted_values = [&](const uint64_t* k, const std::vector<uint32_t>& at) {
+    std::vector<double> v(m);
+    for (size_t i = 0; i < m; ++i) v[i] = vals[at[i]];
+    for (size_t i = 0; i < m;) {
+      size_t e = i + 1;
+      while (e < m && equal(k + (size_t)at[i] * K, k + (size_t)at[e] * K)) ++e;
+      if (e - i > 1) std::sort(v.begin() + (long)i, v.begin() + (long)e);
+      i = e;
     }
-    if (img.size() != base.size()) return false;
-    for (auto& kv : img) {
-      auto it = base.find(kv.first);
-      if (it == base.end() || it->second.size() != kv.second.size()) return false;
-      std::sort(kv.second.begin(), kv.second.end());
-      for (size_t t = 0; t < kv.second.size(); ++t) {
-        double a = kv.second[t], b = it->second[t];
-        if (std::fabs(a - b) > rel_tol * std::max(1.0, std::max(std::fabs(a), std::fabs(b))))
-          return false;
-      }
+    return v;
+  };
+  const std::vector<std::vector<int>> gens = generators(group, n);
+  if (gens.empty()) return true;
+  const std::vector<uint32_t> base = key_order(keys, m, K);
+  const std::vector<double> base_v = sorted_values(keys, base);
+  std::vector<uint64_t> img(m * (size_t)K);
+  for (const auto& g : gens) {
+    for (size_t i = 0; i < m; ++i) {
+      const uint64_t* k = keys + i * K;
+      permute_string(k, k + W, n, W, g, &img[i * K], &img[i * K + W]);
+    }
+    const std::vector<uint32_t> at = key_order(img.data(), m, K);
+    const std::vector<double> v = sorted_values(img.data(), at);
+    for (size_t i = 0; i < m; ++i) {
+      if (!equal(keys + (size_t)base[i] * K, &img[(size_t)at[i] * K])) return false;
+      const double a = v[i], b = base_v[i];
+      if (std::fabs(a - b) > rel_tol * std::max(1.0, std::max(std::fabs(a), std::fabs(b)))) return false;
     }
   }
   return true;
+}
+
+inline bool multiset_invariant(int group, int n, int W, const std::vector<HKey>& keys,
+                               const std::vector<double>& vals, double rel_tol) {
+  std::vector<uint64_t> flat;
+  flat.reserve(keys.size() * 2 * W);
+  for (const HKey& k : keys) flat.insert(flat.end(), k.begin(), k.end());
+  return multiset_invariant(group, n, W, flat.data(), vals.data(), keys.size(), rel_tol);
 }
 
 inline bool bloch_invariant(int group, int n, const double* bloch) {
