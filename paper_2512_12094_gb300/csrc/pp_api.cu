@@ -432,7 +432,7 @@ pp_status compact_into(pp_ctx* c, int dst, double extra_eps, int extra_wmax) {
   PP_CUDA(cudaMemsetAsync(d.index, 0, (size_t)d.icap * 8, c->stream));
   PP_TRY(ctl_prepare_insert(c, 0));
   if (c->batched) {
-    PP_CUDA(launch_compact_batched(c->W, grid_for(c, c->n_terms, 4), c->stream,
+    PP_CUDA(launch_compact_batched(c->W, grid_for(c, c->n_terms * 8, 1), c->stream,
                                    desc_of(c, c->buf[c->active]), c->n_terms, desc_of(c, d), 1,
                                    extra_eps, extra_wmax, c->d_ctl));
   } else {
@@ -1183,7 +1183,7 @@ pp_status restore_snapshot(pp_ctx* c, const Buf& s, uint64_t n) {
     src.index = nullptr;
     src.imask = 0;
     if (c->batched) {
-      PP_CUDA(launch_compact_batched(c->W, grid_for(c, n, 4), c->stream, src, n, desc_of(c, d), 1,
+      PP_CUDA(launch_compact_batched(c->W, grid_for(c, n * 8, 1), c->stream, src, n, desc_of(c, d), 1,
                                      0.0, -1, c->d_ctl));
     } else {
       PP_CUDA(launch_compact(c->W, grid_for(c, n, 4), c->stream, src, n, desc_of(c, d), 1,
@@ -2078,7 +2078,7 @@ pp_status pp_export(pp_ctx* c, int64_t capacity, uint64_t* x, uint64_t* z, doubl
   // active table stays active, and so do its occupancy masks)
   PP_TRY(ctl_prepare_insert(c, 0, false));
   if (c->batched) {
-    PP_CUDA(launch_compact_batched(W, grid_for(c, c->n_terms, 4), c->stream,
+    PP_CUDA(launch_compact_batched(W, grid_for(c, c->n_terms * 8, 1), c->stream,
                                    desc_of(c, c->buf[c->active]), c->n_terms, desc_of(c, d), 0,
                                    0.0, -1, c->d_ctl));
   } else {

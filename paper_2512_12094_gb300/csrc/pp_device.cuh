@@ -647,37 +647,32 @@ __device__ __forceinline__ uint64_t rot_bits(uint64_t m, int s, int n, uint64_t 
   return s == 0 ? m : (((m << s) | (m >> (n - s))) & nmask);
 }
 
+// Compared on the masks: the highest site where two strings differ decides.
+// (Spreading every translation into a 128-bit digit integer was ALU-bound at some
+// 200 instructions each; the merge of a 5 x 6 torus layer of 1.2e7 strings took
+// 3.0 ms, see merge_insert_kernel for what it takes now.)
 __device__ __forceinline__ void canon_torus_w1(Key<1>& k, int n, int lx) {
-  typedef unsigned __int128 u128;
   const int ly = n / lx;
   const uint64_t nmask = (n == 64) ? ~0ull : ((1ull << n) - 1ull);
   const uint64_t x = k.x(0), z = k.z(0);
-  auto dig = [](uint64_t xx, uint64_t zz) {
-    return (u128)digits32((uint32_t)xx, (uint32_t)zz) |
-           ((u128)digits32((uint32_t)(xx >> 32), (uint32_t)(zz >> 32)) << 64);
-  };
-  u128 best = dig(x, z);
-  uint64_t bx = x, bz = z;
+  Key<1> best = k;
+  // first column of every row, from which the masks of the first columns follow
+  uint64_t col0 = 0;
+  for (int y = 0; y < ly; ++y) col0 |= 1ull << (lx * y);  // lx * y < n <= 64
+  uint64_t low = nmask;  // columns [0, lx - dx): they move up by dx, the rest wrap down
   for (int dx = 0; dx < lx; ++dx) {
-    // columns [0, lx - dx) move up by dx, the rest wrap down by lx - dx
-    uint64_t low = 0;
-    const uint64_t row = (lx - dx >= 64) ? ~0ull : ((1ull << (lx - dx)) - 1ull);
-    for (int y = 0; y < ly; ++y) low |= row << (lx * y);  // lx * y < n <= 64
     const uint64_t high = nmask & ~low;
     const uint64_t sx = dx == 0 ? x : (((x & low) << dx) | ((x & high) >> (lx - dx)));
     const uint64_t sz = dx == 0 ? z : (((z & low) << dx) | ((z & high) >> (lx - dx)));
     for (int dy = 0; dy < ly; ++dy) {
-      const uint64_t tx = rot_bits(sx, lx * dy, n, nmask), tz = rot_bits(sz, lx * dy, n, nmask);
-      const u128 v = dig(tx, tz);
-      if (v < best) {
-        best = v;
-        bx = tx;
-        bz = tz;
-      }
+      Key<1> t;
+      t.x(0) = rot_bits(sx, lx * dy, n, nmask);
+      t.z(0) = rot_bits(sz, lx * dy, n, nmask);
+      if (key_less<1>(t, best)) best = t;
     }
+    low &= ~(col0 << (lx - 1 - dx));
   }
-  k.x(0) = bx;
-  k.z(0) = bz;
+  k = best;
 }
 
 template <int W>

@@ -858,51 +858,67 @@ __global__ void __launch_bounds__(kDT, 2)
   }
 }
 
-// After the last phase (one warp): the statistics every path keeps, and the
+// After the last phase (one block): the statistics every path keeps, and the
 // table's size.  A failed layer raises the stall flag instead, which holds off
 // what is queued behind it.
-__global__ void phase_end_kernel(DevCtl* ctl, PhaseAcc acc, unsigned n_gates) {
-  const int lane = threadIdx.x;
+__global__ void __launch_bounds__(kBlock) phase_end_kernel(DevCtl* ctl, PhaseAcc acc, unsigned n_gates) {
+  __shared__ long long s_w[kBlock / 32], s_sum[4];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (acc.st->fail) {
-    if (lane == 0) ctl->stall = acc.st->fail;
+    if (tid == 0) ctl->stall = acc.st->fail;
     return;
   }
+  if (tid < 4) s_sum[tid] = 0;
   long long run = (long long)acc.st->live0, upd = 0, skipped = 0, n_skip = 0, sum_ac = 0;
-  for (unsigned g0 = 0; g0 < n_gates; g0 += 32) {
-    const unsigned g = g0 + lane;
-    const long long d = g < n_gates ? acc.delta[g] : 0;
+  for (unsigned g0 = 0; g0 < n_gates; g0 += kBlock) {
+    const unsigned g = g0 + tid;
+    const bool on = g < n_gates;
+    const long long d = on ? acc.delta[g] : 0;
+    const unsigned long long ac = on ? acc.ac[g] : 0ull;
+    const unsigned touch = on ? acc.touch[g] : 0u, seen = on ? acc.seen[g] : 0u;
     long long x = d;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const long long y = __shfl_up_sync(kFull, x, o);
       if (lane >= o) x += y;
     }
-    if (g < n_gates) {
-      const long long live = run + x - d;  // entering gate g
+    __syncthreads();
+    if (lane == 31) s_w[warp] = x;
+    __syncthreads();
+    long long before = run, all = run;
+    for (int w = 0; w < kBlock / 32; ++w) {
+      if (w < warp) before += s_w[w];
+      all += s_w[w];
+    }
+    if (on) {
+      const long long live = before + x - d;  // entering gate g
       upd += live;
-      sum_ac += (long long)acc.ac[g];
-      if (!acc.touch[g]) {
+      sum_ac += (long long)ac;
+      if (!touch) {
         skipped += live;
         ++n_skip;
       }
-      const double seen = (double)acc.ac[g] + (double)kSample * acc.seen[g];
-      acc.activity[g] = live > 0 ? (float)(seen / (double)live) : 0.0f;
+      acc.activity[g] = live > 0 ? (float)(((double)ac + (double)kSample * seen) / (double)live) : 0.0f;
     }
-    run += __shfl_sync(kFull, x, 31);
+    run = all;
   }
   upd = warp_sum(upd);
   skipped = warp_sum(skipped);
   n_skip = warp_sum(n_skip);
   sum_ac = warp_sum(sum_ac);
+  __syncthreads();
   if (lane == 0) {
-    upd += acc.st->upd;
-    sum_ac += (long long)acc.st->ac;
-    skipped += acc.st->skipped;
-    ctl->updates += (double)upd;
+    const long long v[4] = {upd, skipped, n_skip, sum_ac};
+    for (int k = 0; k < 4; ++k)
+      if (v[k]) atomicAdd(reinterpret_cast<unsigned long long*>(&s_sum[k]), (unsigned long long)v[k]);
+  }
+  __syncthreads();
+  if (tid == 0) {
+    ctl->updates += (double)(s_sum[0] + acc.st->upd);
     ctl->gates_done += n_gates;
-    ctl->ac_total += (unsigned long long)sum_ac;
-    ctl->skipped_updates += (double)skipped;
-    ctl->gates_skipped += (unsigned long long)n_skip;
+    ctl->ac_total += (unsigned long long)s_sum[3] + acc.st->ac;
+    ctl->skipped_updates += (double)(s_sum[1] + acc.st->skipped);
+    ctl->gates_skipped += (unsigned long long)s_sum[2];
     ctl->n_terms = ctl->n_next;
     ctl->n_live = (long long)ctl->n_next;
     ctl->after_terms = ctl->n_next;
@@ -1006,7 +1022,7 @@ cudaError_t launch_phase(int P, int warps, cudaStream_t s, const PhaseBuckets& i
 }
 
 cudaError_t launch_phase_end(cudaStream_t s, DevCtl* ctl, const PhaseAcc& acc, unsigned n_gates) {
-  phase_end_kernel<<<1, 32, 0, s>>>(ctl, acc, n_gates);
+  phase_end_kernel<<<1, kBlock, 0, s>>>(ctl, acc, n_gates);
   return cudaGetLastError();
 }
 
