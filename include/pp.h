@@ -299,7 +299,8 @@ pp_status pp_set_budget(pp_ctx* ctx, size_t mem_budget_bytes);
  * same time only if the fractions of those running together add up to at
  * most 1: then every launch fits beside the others.  A launch over a small
  * table uses fewer blocks than its fraction allows.  Takes effect at the
- * context's next layer.  PP_ERR_ARG for a fraction outside (0, 1]. */
+ * context's next layer; layers applied as phases (see layer_kernel) have no
+ * blocks that wait for one another and are not limited.  PP_ERR_ARG for a fraction outside (0, 1]. */
 pp_status pp_set_grid_fraction(pp_ctx* ctx, double fraction);
 
 /* Wait for all work queued by ctx. */

@@ -1277,7 +1277,7 @@ PhaseSizes phase_sizes(const pp_ctx* c, size_t G, size_t P) {
     // rows of the phases between, and of classes larger than shared memory
     const size_t row = (size_t)c->B * c->esize;
     z.rows = P >= 2 ? align256(c->buf[c->active].cap * row) : 0;
-    z.spill = align256(rows_launch(P32, c->B, (int)c->esize, c->sms, c->grid_frac).spill_rows * row);
+    z.spill = align256(rows_launch(P32, c->B, (int)c->esize, c->sms).spill_rows * row);
     z.bytes += z.rows + z.spill;
   }
   return z;
@@ -1323,7 +1323,10 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   const size_t need = z.bytes;
   const double est = z.est;
   const int P32 = phase_words(c->n);
-  const int warps = std::max(4, (int)std::floor(c->sms * phase_warps_per_sm() * c->grid_frac));
+  // the whole GPU whatever the context's grid fraction: their blocks wait for
+  // nothing, so launches of other contexts need no room beside them (24 served
+  // jobs: 24.5 ms, 26.2 on their fractions)
+  const int warps = c->sms * phase_warps_per_sm();
   auto al = align256;
   const size_t clear = z.clear;
   if (nb >= (1ull << 26) || need > kPhaseBytesMax) return PP_OK;
@@ -1395,7 +1398,7 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   buckets[0].cnt = cnt;
   const int dgrid = (int)std::min<uint64_t>((T + kBlock - 1) / kBlock, (uint64_t)c->sms * 8);
   if (c->batched) {
-    const RowsLaunch L = rows_launch(P32, c->B, (int)c->esize, c->sms, c->grid_frac);
+    const RowsLaunch L = rows_launch(P32, c->B, (int)c->esize, c->sms);
     run(launch_rows_deal(P32, dgrid, c->stream, desc_of(c, c->buf[src]), T, buckets[0], (unsigned)nb,
                          (unsigned)cg, desc(0), ent.d_args, acc));
     const void* from = c->buf[src].rows;

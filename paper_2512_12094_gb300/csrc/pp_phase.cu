@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(kPT, kPBlocks)
   constexpr int W = (P + 1) / 2;
   // set by an earlier kernel of the stream, or by this one: then nothing of the
   // layer is kept
-  if (*reinterpret_cast<const volatile unsigned*>(&acc.st->fail) != 0u) return;
+  if (__syncthreads_or(*reinterpret_cast<const volatile unsigned*>(&acc.st->fail) != 0u)) return;
   const int tid = threadIdx.x, lane = tid & 31;
   const unsigned below = (1u << lane) - 1u;
   PhaseWarp<P>& S = B.warp[tid / 32];
@@ -557,7 +557,7 @@ __global__ void __launch_bounds__(kDT, 2)
                        DevTable dense, DevCtl* ctl, PhaseAcc acc) {
   extern __shared__ __align__(16) unsigned char phase_raw[];
   DenseSmem<P>& S = *reinterpret_cast<DenseSmem<P>*>(phase_raw);
-  if (*reinterpret_cast<const volatile unsigned*>(&acc.st->fail) != 0u) return;
+  if (__syncthreads_or(*reinterpret_cast<const volatile unsigned*>(&acc.st->fail) != 0u)) return;
   const int tid = threadIdx.x, lane = tid & 31;
   const unsigned below = (1u << lane) - 1u;
   const uint64_t eps_bits = rule.eps_bits;

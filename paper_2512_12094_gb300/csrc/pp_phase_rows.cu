@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(256)
   RowsSmem<P>& S = *reinterpret_cast<RowsSmem<P>*>(phase_raw);
   T* const shared_rows = reinterpret_cast<T*>(phase_raw + (sizeof(RowsSmem<P>) + 15) / 16 * 16);
   T* const spill_rows = spill + (uint64_t)blockIdx.x * kRMembers * B;
-  if (*reinterpret_cast<const volatile unsigned*>(&acc.st->fail) != 0u) return;
+  if (__syncthreads_or(*reinterpret_cast<const volatile unsigned*>(&acc.st->fail) != 0u)) return;
   const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31;
   const uint64_t eb = use_eps ? row_eps_bits<T>(eps) : 0ull;
   load_generators<P>(S.mine, gates, d);
@@ -384,7 +384,7 @@ cudaError_t launch_rows_pt(const RowsLaunch& L, cudaStream_t s, const PhaseBucke
 
 }  // namespace
 
-RowsLaunch rows_launch(int P, int B, int esize, int sms, double fraction) {
+RowsLaunch rows_launch(int P, int B, int esize, int sms) {
   RowsLaunch L;
   L.threads = std::min(256, std::max(64, (B + 31) / 32 * 32));
   const size_t fixed = ((P == 1 ? sizeof(RowsSmem<1>) : sizeof(RowsSmem<2>)) + 15) / 16 * 16;
@@ -394,7 +394,7 @@ RowsLaunch rows_launch(int P, int B, int esize, int sms, double fraction) {
   L.smem_rows = (int)std::min<size_t>(kRMembers, (room - fixed) / row);
   L.smem = fixed + (size_t)L.smem_rows * row;
   const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(8, 226 * 1024 / (L.smem + 1024)));
-  L.grid = std::max(1, (int)(sms * per_sm * fraction));
+  L.grid = sms * per_sm;
   L.spill_rows = (size_t)L.grid * kRMembers;
   return L;
 }
