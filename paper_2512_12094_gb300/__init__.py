@@ -20,7 +20,8 @@ _ROOT = os.path.dirname(_HERE)
 _CSRC = os.path.join(_HERE, "csrc")
 _LIB = os.path.join(_HERE, "libpp.so")
 _SOURCES = ["pp_kernels.cu", "pp_api.cu", "pp_static.cu", "pp_batched.cu", "pp_server.cu",
-            "pp_sort.cu", "pp_phase.cu", "pp_phase_rows.cu"]
+            "pp_sort.cu", "pp_phase.cu", "pp_phase_rows.cu",
+            "pp_merge.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
               "--expt-relaxed-constexpr"]

@@ -1240,6 +1240,12 @@ bool phases_allowed(const pp_ctx* c) {
 // pass per gate costs one and a barrier.
 constexpr int kPhaseMinGates = 3;
 constexpr int kPhaseMax = 64;       // phases of a layer
+// Strings of the input table from which a phased layer's merge goes by buckets.
+// Layers of the 32-site ring take the same with 1024, 8192 and 65536 (16.9 to 17.2
+// ms for 20 of them; 18.5 with the index at every size); below, the merge costs a
+// few launches either way, and the index is of use to a layer the persistent
+// kernel applies next.
+constexpr uint64_t kMergeTerms = 1024;
 constexpr double kRowsFill = 8.0;    // of rows
 constexpr double kDenseFill = 700.0; // strings of a bucket in the expected table, dense classes
 constexpr int kPhaseBits = 10;      // key bits a run that does not commute may touch
@@ -1431,7 +1437,21 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   c->launches += (int64_t)P + 3;
   if (e != cudaSuccess) return release(cuda_fail(e, "phase launch"));
   c->index_ok = false;  // of either table from here on, until the merge has rebuilt one
-  if (merge) {
+  // The merge goes back into the source's table: by buckets (in the phases'
+  // scratch, which it needs less of) where the table is not tiny and the orbits
+  // are not S_n's, otherwise by the hash index.
+  MergeBuckets mb = merge_buckets(c->n, (uint64_t)z.est, c->sms);
+  const bool by_buckets = merge && group_kind(c->cfg.symmetry) != PP_SYM_SN &&
+                          c->cfg.merge_method == PP_MERGE_HASH && T >= kMergeTerms &&
+                          mb.bytes <= need - al(clear) - al(G * 4);
+  if (by_buckets) {
+    place_merge_buckets(mb, c->n, scratch + al(clear) + al(G * 4));
+    run(launch_merge_buckets(mb, c->n, c->cfg.symmetry, c->stream, desc_of(c, c->buf[dst]), 0,
+                             &c->d_ctl->n_terms, 0, c->cfg.coeff_eps, desc_of(c, c->buf[src]), c->d_ctl,
+                             c->sms, 1));
+    c->launches += 4;
+    if (e != cudaSuccess) return release(cuda_fail(e, "merge launch"));
+  } else if (merge) {
     const pp_status st = queue_merge(c, c->cfg.symmetry, dst, src);
     if (st != PP_OK) return release(st);
   }
@@ -1447,6 +1467,17 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   release(PP_OK);
   if (st == PP_OK) st = check_device_error(c);
   if (st != PP_OK) return st;
+  if (c->h_ctl->stall == kMergeFull) {
+    // the gates are done, in the other table; their merge is left to the index
+    c->phase_fails = 0;
+    c->last_growth = (double)c->h_ctl->after_terms / (double)T;
+    c->n_terms = c->h_ctl->n_terms;
+    c->n_live = c->h_ctl->n_live;
+    c->live_known = true;
+    PP_TRY(activate(c, dst));
+    *done = true;
+    return merge_active(c, c->cfg.symmetry);
+  }
   if (const unsigned why = c->h_ctl->stall) {
     // given up: the input table is whole (its index may not be).  Next time
     // with finer phases or more buckets, and after ever longer waits.
@@ -1476,6 +1507,7 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   if (want_activity) ent.activity.assign(c->h_activity, c->h_activity + G);
   if (merge) {
     PP_TRY(finish_queued_merge(c, src));
+    c->index_ok = !by_buckets;
   } else {
     c->n_terms = c->h_ctl->n_terms;
     c->n_live = c->h_ctl->n_live;
@@ -2194,6 +2226,66 @@ pp_status pp_canonical_keys(int n_qubits, int symmetry, int64_t m, const uint64_
   return PP_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// Whether a list is merged by buckets: at every length (Z_32, microseconds a call
+// by buckets and by the index: 44 and 73 for 2048 terms, 56 and 99 for 65536,
+// 132 and 197 for a million), except over S_n, whose orbits may all be one, and
+// where the list is longer than there are strings, so that most are repeats.
+bool list_by_buckets(int n, int symmetry, int64_t m) {
+  return group_kind(symmetry) != PP_SYM_SN && (n >= 31 || m <= ((int64_t)1 << (2 * n)));
+}
+
+// pp_merge_terms by buckets; PP_ERR_CAPACITY (nothing reported) when a bucket
+// overflows or its scratch is not to be had.
+pp_status merge_list_by_buckets(int n, int symmetry, int64_t m, const uint64_t* keys_in,
+                                const double* coef_in, uint64_t* keys_out, double* coef_out,
+                                int64_t* m_out, cudaStream_t s) {
+  // the source has to outlive a failure: not where the results are written over it
+  const size_t kb = (size_t)m * 16 * ((n + 63) / 64), cb = (size_t)m * 8;
+  auto apart = [](const void* a, const void* b, size_t bytes) {
+    const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+    return x + bytes <= y || y + bytes <= x;
+  };
+  if (!apart(keys_in, keys_out, kb) || !apart(coef_in, coef_out, cb)) return PP_ERR_CAPACITY;
+  const int sms = std::max(1, device_sm_count());
+  MergeBuckets mb = merge_buckets(n, (uint64_t)m, sms);
+  if (mb.bytes > kPhaseBytesMax) return PP_ERR_CAPACITY;
+  const size_t ctl_bytes = (sizeof(DevCtl) + 255) / 256 * 256;
+  unsigned char* scratch = nullptr;
+  if (cudaMallocAsync((void**)&scratch, ctl_bytes + mb.bytes, s) != cudaSuccess) {
+    cudaGetLastError();
+    return PP_ERR_CAPACITY;
+  }
+  DevCtl* ctl = reinterpret_cast<DevCtl*>(scratch);
+  place_merge_buckets(mb, n, scratch + ctl_bytes);
+  DevTable src = {}, dst = {};
+  src.keys = const_cast<uint64_t*>(keys_in);
+  src.coef = const_cast<double*>(coef_in);
+  src.cap = (uint64_t)m;
+  dst.keys = keys_out;
+  dst.coef = coef_out;
+  dst.cap = (uint64_t)m;
+  DevCtl h;
+  memset(&h, 0, sizeof(h));
+  cudaError_t e = cudaMemsetAsync(ctl, 0, sizeof(DevCtl), s);
+  if (e == cudaSuccess)
+    e = launch_merge_buckets(mb, n, symmetry, s, src, (uint64_t)m, nullptr, 0, 0.0, dst, ctl, sms, 0);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  cudaFreeAsync(scratch, s);
+  if (e != cudaSuccess) return cuda_fail(e, "pp_merge_terms");
+  if (h.stall) return PP_ERR_CAPACITY;
+  *m_out = (int64_t)h.n_next;
+  return PP_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 pp_status pp_merge_terms(int n_qubits, int symmetry, int64_t m, const uint64_t* keys_in,
                          const double* coef_in, uint64_t* keys_out, double* coef_out,
                          int64_t* m_out, void* stream) {
@@ -2206,6 +2298,11 @@ pp_status pp_merge_terms(int n_qubits, int symmetry, int64_t m, const uint64_t* 
   if (m == 0) return PP_OK;
   cudaStream_t s = (cudaStream_t)stream;
   const int W = (n_qubits + 63) / 64;
+  if (list_by_buckets(n_qubits, symmetry, m)) {
+    const pp_status st = merge_list_by_buckets(n_qubits, symmetry, m, keys_in, coef_in, keys_out, coef_out,
+                                               m_out, s);
+    if (st != PP_ERR_CAPACITY) return st;  // too many equal strings: by the hash index
+  }
   const uint64_t icap = next_pow2(2 * (uint64_t)m);
   uint64_t* index = nullptr;
   DevCtl* ctl = nullptr;

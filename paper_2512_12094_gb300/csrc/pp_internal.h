@@ -288,6 +288,26 @@ cudaError_t launch_phase(int P, int warps, cudaStream_t s, const PhaseBuckets& i
                          const PhaseBuckets& out, unsigned nb, unsigned cg, const PhaseDesc& d,
                          const PhaseDesc& next, const GateArgs* gates, const PhaseRule& rule,
                          const DevTable& dense, DevCtl* ctl, const PhaseAcc& acc);
+// Merge by buckets (pp_merge.cu), any group but S_n (whose orbits may all be one):
+// representatives of src (count entries, or *count_dev) added up into dst from
+// its first entry on, n_next counting them; entries that eps truncates are
+// dropped.  n_terms and n_live follow, or ctl->stall becomes kMergeFull and the
+// source is to be merged by the hash index.  guarded: nothing happens where
+// stall or error is set.
+enum : unsigned { kMergeFull = 8u };
+struct MergeBuckets {
+  PhaseBuckets buckets;
+  unsigned nb, cg;
+  unsigned* fail;  // 64 words ahead of the counters
+  size_t bytes;
+};
+MergeBuckets merge_buckets(int n, uint64_t count, int sms);
+void place_merge_buckets(MergeBuckets& m, int n, void* scratch);
+cudaError_t launch_merge_buckets(const MergeBuckets& m, int n, int group, cudaStream_t s,
+                                 const DevTable& src, uint64_t count,
+                                 const unsigned long long* count_dev, int skip_zero, double eps,
+                                 const DevTable& dst, DevCtl* ctl, int sms, int guarded);
+
 // Batched layers (pp_phase_rows.cu; n <= 64, dense phases only): buckets hold row
 // numbers in place of coefficients.
 struct RowsLaunch {

@@ -95,6 +95,22 @@ __device__ __forceinline__ void st_pkey(uint32_t* keys, uint64_t i, const PKey<P
   }
 }
 
+template <int P>
+__device__ __forceinline__ uint64_t string_hash(const PKey<P>& v, uint32_t seed) {
+  uint32_t a = 0x9E3779B9u ^ seed, b = 0x7F4A7C15u + seed;
+#pragma unroll
+  for (int j = 0; j < P; ++j) {
+    const uint32_t lo = v.w[j], hi = v.w[P + j];
+    a = (a ^ lo) * 0xcc9e2d51u;
+    a = __funnelshift_l(a, a, 15) ^ hi;
+    a *= 0x1b873593u;
+    b = (b ^ hi) * 0x27d4eb2fu;
+    b = __funnelshift_l(b, b, 13) ^ lo;
+    b *= 0x165667b1u;
+  }
+  return ((uint64_t)fmix32(a ^ b) << 32) | fmix32(b + 0x9E3779B9u * a);
+}
+
 // Active gates and class hash of a string in the phase that comes next: the hash
 // of the string with the bits masked out that an active generator touches, or,
 // for a dense phase, of the string reduced by its active generators (where it
@@ -138,18 +154,7 @@ __device__ __forceinline__ void classify(const PKey<P>& K, const NextGens<P>& ne
       v.w[P + j] &= ~(uint32_t)(d.uz[j / 2] >> (32 * (j & 1)));
     }
   }
-  uint32_t a = 0x9E3779B9u ^ act, b = 0x7F4A7C15u + act;
-#pragma unroll
-  for (int j = 0; j < P; ++j) {
-    const uint32_t lo = v.w[j], hi = v.w[P + j];
-    a = (a ^ lo) * 0xcc9e2d51u;
-    a = __funnelshift_l(a, a, 15) ^ hi;
-    a *= 0x1b873593u;
-    b = (b ^ hi) * 0x27d4eb2fu;
-    b = __funnelshift_l(b, b, 13) ^ lo;
-    b *= 0x165667b1u;
-  }
-  h = ((uint64_t)fmix32(a ^ b) << 32) | fmix32(b + 0x9E3779B9u * a);
+  h = string_hash<P>(v, act);
 }
 
 // Append a string to its bucket of the next phase.
