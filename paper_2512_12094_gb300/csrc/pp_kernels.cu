@@ -867,6 +867,110 @@ __global__ void __launch_bounds__(kBlock)
   }
 }
 
+// The Z_n average in a product state, four sites at a time: the product over the
+// letters of sites q .. q + 3 (mod n) for each of the 256 sets of letters is kept
+// in shared memory, so a translation of a string takes one factor per window of
+// four sites that it touches, each window starting at the first letter left over,
+// in the place of one per letter.
+//
+// Bound by the FP64 pipe either way, products and sums per string and
+// translation: as many as windows here, 1 + weight letter by letter.  975 thousand
+// strings of weight 8 on 32 sites: 369 us, 513 letter by letter.  A block of
+// 32 warps an SM shares one table (64 KB at 32 sites), filled from one of pairs
+// of sites with a product per entry: n * 8 of a warp, as much as 64 to 128 strings
+// of weight one take, hence the least number of strings in launch_overlap.
+constexpr int kOvThreads = 1024;
+constexpr int kOvStrings = 2048;  // an SM, at least
+constexpr int kOvSites = 104;     // whose tables fit in shared memory
+inline size_t overlap_blocks_smem(int n) { return (size_t)n * (256 + 16) * sizeof(double); }
+
+template <int W>
+__global__ void __launch_bounds__(kOvThreads)
+    overlap_zn_blocks_kernel(const uint64_t* __restrict__ keys, const double* __restrict__ coef,
+                             uint64_t count, OverlapArgs a, double* partials) {
+  extern __shared__ __align__(16) double ov_table[];  // [n][256], then [n][16] of pairs
+  __shared__ double s_acc[kOvThreads / 32];
+  const int n = a.n;
+  double* const pairs = ov_table + n * 256;
+  // a set of letters of two sites: x bits 0, 1 and z bits 2, 3; of four: x 0-3, z 4-7
+  for (int i = threadIdx.x; i < n * 16; i += kOvThreads) {
+    double v = 1.0;
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int xb = (i >> b) & 1, zb = (i >> (2 + b)) & 1;
+      if (xb | zb) v *= a.bloch[3 * (((i >> 4) + b) % n) + (xb ? (zb ? 1 : 0) : 2)];
+    }
+    pairs[i] = v;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n * 256; i += kOvThreads) {
+    const int q = i >> 8, x = i & 15, z = (i >> 4) & 15;
+    ov_table[i] = pairs[q * 16 + (x & 3) + (z & 3) * 4] *
+                  pairs[((q + 2) % n) * 16 + (x >> 2) + (z >> 2) * 4];
+  }
+  __syncthreads();
+  double acc = 0.0;
+  const uint64_t stride = (uint64_t)gridDim.x * kOvThreads;
+  for (uint64_t i = (uint64_t)blockIdx.x * kOvThreads + threadIdx.x; i < count; i += stride) {
+    const double c = coef[i];
+    if (c == 0.0) continue;
+    const Key<W> k = ld_key<W>(keys, i);
+    // the first window, whose factor needs no product, and the letters after it
+    uint64_t rest[W];
+    int q0 = -1, set0 = 0;
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+      uint64_t m = k.x(j) | k.z(j);
+      if (q0 < 0 && m) {
+        const int b = __ffsll((long long)m) - 1;
+        m &= ~(15ull << b);
+        q0 = 64 * j + b;
+        set0 = (int)((k.x(j) >> b) & 15ull) + (int)((k.z(j) >> b) & 15ull) * 16;
+      }
+      rest[j] = m;
+    }
+    q0 = max(q0, 0);
+    double sum = 0.0;
+    for (int s = 0; s < n; ++s) {
+      const int qs = q0 - s;
+      double v = ov_table[(qs < 0 ? qs + n : qs) * 256 + set0];
+#pragma unroll
+      for (int j = 0; j < W; ++j) {
+        uint64_t m = rest[j];
+        while (m) {
+          const int b = __ffsll((long long)m) - 1;
+          m &= ~(15ull << b);
+          int q = 64 * j + b - s;
+          q += (q < 0) ? n : 0;
+          v *= ov_table[q * 256 + (int)((k.x(j) >> b) & 15ull) + (int)((k.z(j) >> b) & 15ull) * 16];
+        }
+      }
+      sum += v;
+    }
+    acc += c * (sum / (double)n);
+  }
+  acc = warp_sum(acc);
+  if ((threadIdx.x & 31) == 0) s_acc[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int w = 0; w < kOvThreads / 32; ++w) s += s_acc[w];
+    partials[blockIdx.x] = s;
+  }
+}
+
+template <int W>
+cudaError_t launch_overlap_blocks(int grid, cudaStream_t s, const uint64_t* keys, const double* coef,
+                                  uint64_t count, const OverlapArgs& a, double* partials) {
+  const cudaError_t e = cudaFuncSetAttribute(overlap_zn_blocks_kernel<W>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)overlap_blocks_smem(kOvSites));
+  if (e != cudaSuccess) return e;
+  overlap_zn_blocks_kernel<W><<<grid, kOvThreads, overlap_blocks_smem(a.n), s>>>(keys, coef, count, a,
+                                                                                 partials);
+  return cudaGetLastError();
+}
+
 __global__ void __launch_bounds__(kBlock) reduce_partials_kernel(const double* partials, int m,
                                                                 double* out) {
   __shared__ double s_acc[kBlock / 32];
@@ -1131,8 +1235,19 @@ cudaError_t launch_overlap(int W, int grid, cudaStream_t s, const uint64_t* keys
                            const double* coef, uint64_t count,
                            const unsigned long long* count_dev, const OverlapArgs& a,
                            double* partials, double* out) {
-  PP_DISPATCH_W(W, (overlap_kernel<WW><<<grid, kBlock, 0, s>>>(keys, coef, count, count_dev, a,
-                                                               partials)));
+  // grid: four blocks an SM, which the window form has one of
+  const int sms = std::max(1, grid / 4);
+  if (a.group == 1 && !a.basis && !count_dev && a.n <= kOvSites && W <= 2 &&
+      count >= (uint64_t)sms * kOvStrings) {
+    grid = sms;
+    const cudaError_t e =
+        W == 1 ? launch_overlap_blocks<1>(grid, s, keys, coef, count, a, partials)
+               : launch_overlap_blocks<2>(grid, s, keys, coef, count, a, partials);
+    if (e != cudaSuccess) return e;
+  } else {
+    PP_DISPATCH_W(W, (overlap_kernel<WW><<<grid, kBlock, 0, s>>>(keys, coef, count, count_dev, a,
+                                                                 partials)));
+  }
   reduce_partials_kernel<<<1, kBlock, 0, s>>>(partials, grid, out);
   return cudaGetLastError();
 }
