@@ -433,14 +433,47 @@ __device__ __forceinline__ void zn_take_gap(Mask<W>& cand, int& L, int gap, int 
   if (gap == L) mask_set<W>(cand, s);
 }
 
+// Longest cyclic runs of ones of a one-word mask v that has a zero among its n
+// bits: the positions they start at, and their length L.  c_s marks the windows of
+// s ones, s doubling; the length is then put together from its highest bit down,
+// a window of L ones followed by one of s at a time.  Twelve steps whatever the
+// mask (KIND 0: n <= 32 on the mask written twice, whose windows need no wrap;
+// 1: n == 64; 2: any n).
+template <int KIND>
+__device__ __forceinline__ uint64_t zn_longest_runs(uint64_t v, int n, uint64_t nm, int& L) {
+  auto rot = [&](uint64_t a, int s) {  // 0 <= s < n, or any s if a is 0
+    if constexpr (KIND == 0) return a >> (s & 63);
+    if constexpr (KIND == 1) return (a >> (s & 63)) | (a << ((64 - s) & 63));
+    return ((a >> (s & 63)) | ((a << 1) << ((n - 1 - s) & 63))) & nm;
+  };
+  uint64_t c[6];
+  c[0] = KIND == 0 ? (v | (v << n)) : v;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) c[k + 1] = c[k] & rot(c[k], 1 << k);
+  uint64_t cur = nm;
+  L = 0;
+#pragma unroll
+  for (int k = 5; k >= 0; --k) {
+    const uint64_t t = cur & rot(c[k], L);
+    if (t) {
+      cur = t;
+      L += 1 << k;
+    }
+  }
+  return cur;
+}
+
 // Z_n (Algorithm 2): the translation with the lowest digit integer.  Instead
 // of comparing all n translations, the search keeps only those that can be
 // lowest: the top digit of the lowest one is the smallest digit d present,
 // and the longer the run of d at the top, the lower the integer (a shorter
 // run is followed by a larger digit).  So the candidates put a longest
 // cyclic run of d on the top qubits n-L..n-1, that is, translate by j where
-// j is the site just after the run.  The runs are found in one of two ways,
-// both giving every longest run:
+// j is the site just after the run.  One word finds the runs by doubling
+// windows (zn_longest_runs), which every lane does in the same steps; it is bound
+// by integer instructions either way (five million strings of weight 10 on 64
+// sites: 74 us, 137 when they walked gaps as below).  Several words find them in
+// one of two ways, both giving every longest run:
 //  * few sites differ from d (a low-weight string, d = I): walk the gaps
 //    between consecutive such sites, cyclically; a gap before site s is a
 //    run ending just before s, so j = s;
@@ -480,7 +513,12 @@ __device__ __forceinline__ void canon_zn(Key<W>& k, int n) {
 #pragma unroll
   for (int i = 0; i < W; ++i) cand.w[i] = 0;
   int L = -1;  // length of the longest runs
-  if (n_other <= kZnGapWalk) {
+  if constexpr (W == 1) {
+    const Mask<1> cur = {{n <= 32    ? zn_longest_runs<0>(dm.w[0], n, nm.w[0], L)
+                          : n == 64 ? zn_longest_runs<1>(dm.w[0], n, nm.w[0], L)
+                                    : zn_longest_runs<2>(dm.w[0], n, nm.w[0], L)}};
+    cand = mask_rot<1>(cur, n - L, n, nm);  // bit p of cur -> bit (p + L) mod n
+  } else if (n_other <= kZnGapWalk) {
     int first = -1, prev = -1;
 #pragma unroll
     for (int i = 0; i < W; ++i) {
@@ -650,7 +688,7 @@ __device__ __forceinline__ uint64_t rot_bits(uint64_t m, int s, int n, uint64_t 
 // Compared on the masks: the highest site where two strings differ decides.
 // (Spreading every translation into a 128-bit digit integer was ALU-bound at some
 // 200 instructions each; the merge of a 5 x 6 torus layer of 1.2e7 strings took
-// 3.0 ms, see merge_insert_kernel for what it takes now.)
+// 3.0 ms; the merges of seven layers took 8.0 ms together, 2.4 this way.)
 __device__ __forceinline__ void canon_torus_w1(Key<1>& k, int n, int lx) {
   const int ly = n / lx;
   const uint64_t nmask = (n == 64) ? ~0ull : ((1ull << n) - 1ull);
