@@ -1445,7 +1445,7 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
                           c->cfg.merge_method == PP_MERGE_HASH && T >= kMergeTerms &&
                           mb.bytes <= need - al(clear) - al(G * 4);
   if (by_buckets) {
-    place_merge_buckets(mb, c->n, scratch + al(clear) + al(G * 4));
+    place_merge_buckets(mb, scratch + al(clear) + al(G * 4));
     run(launch_merge_buckets(mb, c->n, c->cfg.symmetry, c->stream, desc_of(c, c->buf[dst]), 0,
                              &c->d_ctl->n_terms, 0, c->cfg.coeff_eps, desc_of(c, c->buf[src]), c->d_ctl,
                              c->sms, 1));
@@ -2260,7 +2260,7 @@ pp_status merge_list_by_buckets(int n, int symmetry, int64_t m, const uint64_t* 
     return PP_ERR_CAPACITY;
   }
   DevCtl* ctl = reinterpret_cast<DevCtl*>(scratch);
-  place_merge_buckets(mb, n, scratch + ctl_bytes);
+  place_merge_buckets(mb, scratch + ctl_bytes);
   DevTable src = {}, dst = {};
   src.keys = const_cast<uint64_t*>(keys_in);
   src.coef = const_cast<double*>(coef_in);

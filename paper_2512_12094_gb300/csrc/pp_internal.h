@@ -296,13 +296,14 @@ cudaError_t launch_phase(int P, int warps, cudaStream_t s, const PhaseBuckets& i
 // stall or error is set.
 enum : unsigned { kMergeFull = 8u };
 struct MergeBuckets {
-  PhaseBuckets buckets;
-  unsigned nb, cg;
-  unsigned* fail;  // 64 words ahead of the counters
+  unsigned nb, cg;  // buckets, and their room
+  unsigned* fail;   // 64 words ahead of the counters
+  unsigned* cnt;
+  ulonglong2* rec;  // key and coefficient of a string, (P + 2) / 2 units
   size_t bytes;
 };
 MergeBuckets merge_buckets(int n, uint64_t count, int sms);
-void place_merge_buckets(MergeBuckets& m, int n, void* scratch);
+void place_merge_buckets(MergeBuckets& m, void* scratch);
 cudaError_t launch_merge_buckets(const MergeBuckets& m, int n, int group, cudaStream_t s,
                                  const DevTable& src, uint64_t count,
                                  const unsigned long long* count_dev, int skip_zero, double eps,

@@ -4,12 +4,13 @@
 // Every string is mapped to its representative and dealt into a bucket by the
 // representative's hash, so equal ones meet in one bucket; a block takes a bucket
 // into shared memory, adds equal strings up there and appends what truncation
-// keeps to the destination.  Two passes over the table (32 bytes a string, half
-// of it scattered) in the place of one with three random 32-byte sectors and an
-// atomic per string, and no index to clear (8 to 16 bytes per entry of capacity).
-// 1.95 million strings of 32 sites into 975 thousand under Z_n: 92 us dealt (of
-// which the representatives take most) and 50 us merged, where the index took
-// 0.35 ms with its clearing.
+// keeps to the destination.  Two passes over the table, one of them scattered, a
+// sector a string, in the place of one with three random sectors and an atomic
+// per string, and no index to clear (8 to 16 bytes per entry of capacity).
+// 1.95 million strings of 32 sites into 975 thousand under Z_n: 65 us dealt (82
+// with key, coefficient and hash in arrays of their own) and 44 us merged, where
+// the index took 0.35 ms with its clearing.  Bound by the atomics and scattered
+// sectors of the deal, and by the probes in shared memory after it.
 //
 // A bucket larger than a block's room is done in parts, split by further bits of
 // the hash.  A full bucket, or more equal strings than a block holds, raises
@@ -35,6 +36,38 @@ struct MergeSmem {
   unsigned long long out_base;
 };
 
+// A string in its bucket: key words and coefficient in units of 16 bytes, so that
+// it is scattered in the fewest sectors (one of 32 bytes up to 64 sites).
+template <int P>
+__device__ __forceinline__ void st_rec(ulonglong2* to, uint64_t i, const PKey<P>& k, double c) {
+  constexpr int U = (P + 2) / 2;
+  uint64_t r[2 * U];
+  r[2 * U - 1] = 0ull;
+#pragma unroll
+  for (int j = 0; j < P; ++j) r[j] = (uint64_t)k.w[2 * j] | ((uint64_t)k.w[2 * j + 1] << 32);
+  r[P] = (uint64_t)__double_as_longlong(c);
+#pragma unroll
+  for (int j = 0; j < U; ++j) to[i * U + j] = make_ulonglong2(r[2 * j], r[2 * j + 1]);
+}
+
+template <int P>
+__device__ __forceinline__ double ld_rec(const ulonglong2* from, uint64_t i, PKey<P>& k) {
+  constexpr int U = (P + 2) / 2;
+  uint64_t r[2 * U];
+#pragma unroll
+  for (int j = 0; j < U; ++j) {
+    const ulonglong2 v = from[i * U + j];
+    r[2 * j] = v.x;
+    r[2 * j + 1] = v.y;
+  }
+#pragma unroll
+  for (int j = 0; j < P; ++j) {
+    k.w[2 * j] = (uint32_t)r[j];
+    k.w[2 * j + 1] = (uint32_t)(r[j] >> 32);
+  }
+  return __longlong_as_double((long long)r[P]);
+}
+
 __device__ __forceinline__ bool merge_off(const DevCtl* ctl, const unsigned* fail, int guarded) {
   return (guarded && queued_layer_stopped(ctl)) || *reinterpret_cast<const volatile unsigned*>(fail) != 0u;
 }
@@ -55,10 +88,10 @@ template <int P, int G>
 __global__ void __launch_bounds__(kBlock)
     merge_deal_kernel(const uint64_t* __restrict__ keys, const double* __restrict__ coef,
                       uint64_t count, const unsigned long long* count_dev, int skip_zero, int n, int lx,
-                      PhaseBuckets out, unsigned nb, unsigned cg, unsigned* fail, const DevCtl* ctl,
+                      MergeBuckets out, const DevCtl* ctl,
                       int guarded) {
   constexpr int W = (P + 1) / 2;
-  if (merge_off(ctl, fail, guarded)) return;
+  if (merge_off(ctl, out.fail, guarded)) return;
   const uint64_t T = count_dev ? *count_dev : count;
   unsigned bad = 0;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -73,27 +106,31 @@ __global__ void __launch_bounds__(kBlock)
       k.w[j] = (uint32_t)(K.x(j / 2) >> (32 * (j & 1)));
       k.w[P + j] = (uint32_t)(K.z(j / 2) >> (32 * (j & 1)));
     }
-    deal<P>(out, nb, cg, k, c, 0u, string_hash<P>(k, 0u), bad);
+    const unsigned b = (unsigned)(((string_hash<P>(k, 0u) >> 32) * (uint64_t)out.nb) >> 32);
+    const unsigned p = atomicAdd(out.cnt + b, 1u);
+    if (p < out.cg)
+      st_rec<P>(out.rec, (uint64_t)b * out.cg + p, k, c);
+    else
+      bad = 1;
   }
-  if (bad) atomicOr(fail, kMergeFull);
+  if (bad) atomicOr(out.fail, kMergeFull);
 }
 
 template <int P>
 __global__ void __launch_bounds__(kMT)
-    merge_bucket_kernel(PhaseBuckets in, unsigned nb, unsigned cg, double eps, DevTable dst, unsigned* fail,
-                        DevCtl* ctl, int guarded) {
+    merge_bucket_kernel(MergeBuckets in, double eps, DevTable dst, DevCtl* ctl, int guarded) {
   extern __shared__ __align__(16) unsigned char merge_raw[];
   MergeSmem<P>& S = *reinterpret_cast<MergeSmem<P>*>(merge_raw);
   constexpr int C = MergeSmem<P>::C, W = (P + 1) / 2;
-  if (__syncthreads_or(merge_off(ctl, fail, guarded))) return;  // the whole block or none of it
+  if (__syncthreads_or(merge_off(ctl, in.fail, guarded))) return;  // the whole block or none of it
   const int tid = threadIdx.x, lane = tid & 31;
   const unsigned below = (1u << lane) - 1u;
   unsigned bad = 0;
   OccAcc<W> occ;
-  for (unsigned b = blockIdx.x; b < nb; b += gridDim.x) {
-    const int cnt = (int)min(in.cnt[b], cg);
+  for (unsigned b = blockIdx.x; b < in.nb; b += gridDim.x) {
+    const int cnt = (int)min(in.cnt[b], in.cg);
     if (cnt == 0) continue;
-    const uint64_t base = (uint64_t)b * cg;
+    const uint64_t base = (uint64_t)b * in.cg;
     int s0 = 0;  // parts, as in phase_kernel
     while ((cnt >> s0) > C * 7 / 8) ++s0;
     int s = s0;
@@ -108,14 +145,20 @@ __global__ void __launch_bounds__(kMT)
       __syncthreads();
       for (int i0 = 0; i0 < cnt; i0 += kMT) {
         const int i = i0 + tid;
-        const bool mine = i < cnt && (in.meta[base + i].y & ((1u << s) - 1u)) == id;
+        PKey<P> K;
+        double c = 0.0;
+        bool mine = i < cnt;
+        if (mine) {
+          c = ld_rec<P>(in.rec, base + i, K);
+          if (s > 0) mine = ((unsigned)string_hash<P>(K, 0u) & ((1u << s) - 1u)) == id;
+        }
         const unsigned bal = __ballot_sync(kFull, mine);
         int p = 0;
         if (lane == 0 && bal) p = atomicAdd(&S.n, __popc(bal));
         p = __shfl_sync(kFull, p, 0) + __popc(bal & below);
         if (mine && p < C) {
-          S.key[p] = ld_pkey<P>(in.keys, base + i);
-          S.coef[p] = S.sum[p] = in.coef[base + i];
+          S.key[p] = K;
+          S.coef[p] = S.sum[p] = c;
         }
       }
       __syncthreads();
@@ -186,7 +229,7 @@ __global__ void __launch_bounds__(kMT)
     }
   }
   occ.flush(ctl);
-  if (bad) atomicOr(fail, bad);
+  if (bad) atomicOr(in.fail, bad);
 }
 
 // The merged table's size, or the failure in the stall flag.
@@ -211,14 +254,14 @@ cudaError_t merge_pg(const MergeBuckets& m, cudaStream_t s, const DevTable& src,
   merge_deal_kernel<P, G><<<(int)std::max<uint64_t>(1, std::min<uint64_t>((bound + kBlock - 1) / kBlock,
                                                                           (uint64_t)sms * 8)),
                             kBlock, 0, s>>>(src.keys, src.coef, count, count_dev, skip_zero, n, lx,
-                                            m.buckets, m.nb, m.cg, m.fail, ctl, guarded);
+                                            m, ctl, guarded);
   static const cudaError_t e =
       cudaFuncSetAttribute(merge_bucket_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)sizeof(MergeSmem<P>));
   if (e != cudaSuccess) return e;
   const int per_sm = std::min<int>(8, (int)(226 * 1024 / (sizeof(MergeSmem<P>) + 1024)));
   merge_bucket_kernel<P><<<(int)std::min<uint64_t>(m.nb, (uint64_t)sms * per_sm), kMT,
-                           sizeof(MergeSmem<P>), s>>>(m.buckets, m.nb, m.cg, eps, dst, m.fail, ctl, guarded);
+                           sizeof(MergeSmem<P>), s>>>(m, eps, dst, ctl, guarded);
   merge_end_kernel<<<1, 1, 0, s>>>(m.fail, ctl, guarded);
   return cudaGetLastError();
 }
@@ -234,24 +277,17 @@ MergeBuckets merge_buckets(int n, uint64_t count, int sms) {
   const int P = phase_words(n);
   m.nb = (unsigned)std::max<uint64_t>((uint64_t)sms * 2, (count + 599) / 600);
   m.cg = (unsigned)((2 * count / m.nb + 8 * (uint64_t)n + 256) / 8 * 8);
-  const size_t e = (size_t)m.nb * m.cg;
-  m.bytes = al256((64 + (size_t)m.nb) * 4) + al256(e * 8 * P) + 2 * al256(e * 8);
-  m.fail = nullptr;
+  m.bytes = al256((64 + (size_t)m.nb) * 4) + al256((size_t)m.nb * m.cg * ((P + 2) / 2) * 16);
+  m.fail = m.cnt = nullptr;
+  m.rec = nullptr;
   return m;
 }
 
-void place_merge_buckets(MergeBuckets& m, int n, void* scratch) {
-  const int P = phase_words(n);
-  unsigned char* p = static_cast<unsigned char*>(scratch);
-  const size_t e = (size_t)m.nb * m.cg;
-  m.fail = reinterpret_cast<unsigned*>(p);
-  m.buckets.cnt = m.fail + 64;
-  p += al256((64 + (size_t)m.nb) * 4);
-  m.buckets.keys = reinterpret_cast<uint32_t*>(p);
-  p += al256(e * 8 * P);
-  m.buckets.coef = reinterpret_cast<double*>(p);
-  p += al256(e * 8);
-  m.buckets.meta = reinterpret_cast<uint2*>(p);
+void place_merge_buckets(MergeBuckets& m, void* scratch) {
+  m.fail = static_cast<unsigned*>(scratch);
+  m.cnt = m.fail + 64;
+  m.rec = reinterpret_cast<ulonglong2*>(static_cast<unsigned char*>(scratch) +
+                                        al256((64 + (size_t)m.nb) * 4));
 }
 
 cudaError_t launch_merge_buckets(const MergeBuckets& m, int n, int group, cudaStream_t s,
