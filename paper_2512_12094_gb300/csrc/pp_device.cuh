@@ -433,34 +433,36 @@ __device__ __forceinline__ void zn_take_gap(Mask<W>& cand, int& L, int gap, int 
   if (gap == L) mask_set<W>(cand, s);
 }
 
-// Longest cyclic runs of ones of a one-word mask v that has a zero among its n
-// bits: the positions they start at, and their length L.  c_s marks the windows of
-// s ones, s doubling; the length is then put together from its highest bit down,
-// a window of L ones followed by one of s at a time.  Twelve steps whatever the
-// mask (KIND 0: n <= 32 on the mask written twice, whose windows need no wrap;
-// 1: n == 64; 2: any n).
-template <int KIND>
-__device__ __forceinline__ uint64_t zn_longest_runs(uint64_t v, int n, uint64_t nm, int& L) {
-  auto rot = [&](uint64_t a, int s) {  // 0 <= s < n, or any s if a is 0
-    if constexpr (KIND == 0) return a >> (s & 63);
-    if constexpr (KIND == 1) return (a >> (s & 63)) | (a << ((64 - s) & 63));
-    return ((a >> (s & 63)) | ((a << 1) << ((n - 1 - s) & 63))) & nm;
+// The sites just after the longest cyclic runs of ones of a one-word mask v of n
+// bits, not all ones, and the runs' length L >= 1.  With one of v's zeros turned to
+// the top no run wraps.  Then c_s marks the windows of s ones, s doubling, and the
+// length is put together from its highest bit down, a window of L ones followed by
+// one of s at a time: eleven steps whatever the mask.
+__device__ __forceinline__ uint64_t zn_after_longest_runs(uint64_t v, int n, uint64_t nm, int& L) {
+  auto rot = [&](uint64_t a, int s) {  // toward bit 0, 0 <= s < n
+    return ((a >> s) | ((a << 1) << (n - 1 - s))) & nm;
   };
+  int top = 64 - __clzll((long long)(~v & nm));  // the highest zero goes to bit n - 1
+  top = top == n ? 0 : top;
   uint64_t c[6];
-  c[0] = KIND == 0 ? (v | (v << n)) : v;
+  c[0] = rot(v, top);
 #pragma unroll
-  for (int k = 0; k < 5; ++k) c[k + 1] = c[k] & rot(c[k], 1 << k);
+  for (int k = 0; k < 5; ++k) c[k + 1] = c[k] & (c[k] >> (1 << k));
   uint64_t cur = nm;
   L = 0;
+  if (n > 32 && c[5]) {
+    cur = c[5];
+    L = 32;
+  }
 #pragma unroll
-  for (int k = 5; k >= 0; --k) {
-    const uint64_t t = cur & rot(c[k], L);
+  for (int k = 4; k >= 0; --k) {
+    const uint64_t t = cur & (c[k] >> L);
     if (t) {
       cur = t;
       L += 1 << k;
     }
   }
-  return cur;
+  return rot(cur << L, top == 0 ? 0 : n - top);
 }
 
 // Z_n (Algorithm 2): the translation with the lowest digit integer.  Instead
@@ -469,10 +471,13 @@ __device__ __forceinline__ uint64_t zn_longest_runs(uint64_t v, int n, uint64_t 
 // and the longer the run of d at the top, the lower the integer (a shorter
 // run is followed by a larger digit).  So the candidates put a longest
 // cyclic run of d on the top qubits n-L..n-1, that is, translate by j where
-// j is the site just after the run.  One word finds the runs by doubling
-// windows (zn_longest_runs), which every lane does in the same steps; it is bound
-// by integer instructions either way (five million strings of weight 10 on 64
-// sites: 74 us, 137 when they walked gaps as below).  Several words find them in
+// j is the site just after the run.  One word of which at most
+// half the sites differ from d finds the runs by doubling windows
+// (zn_after_longest_runs), in the same steps on every lane.  Bound by integer
+// instructions: four million strings of 64 sites in 54, 60, 63 and 68 us at
+// weights 4, 8, 12 and 32, where walking gaps took 61, 95 and 127 us and shrinking
+// masks 72 at 32; at weight 48 shrinking takes 63 and doubling 70, which is the
+// reason for the half (at 32 sites they meet at weight 18).  Otherwise they are found in
 // one of two ways, both giving every longest run:
 //  * few sites differ from d (a low-weight string, d = I): walk the gaps
 //    between consecutive such sites, cyclically; a gap before site s is a
@@ -513,12 +518,9 @@ __device__ __forceinline__ void canon_zn(Key<W>& k, int n) {
 #pragma unroll
   for (int i = 0; i < W; ++i) cand.w[i] = 0;
   int L = -1;  // length of the longest runs
-  if constexpr (W == 1) {
-    const Mask<1> cur = {{n <= 32    ? zn_longest_runs<0>(dm.w[0], n, nm.w[0], L)
-                          : n == 64 ? zn_longest_runs<1>(dm.w[0], n, nm.w[0], L)
-                                    : zn_longest_runs<2>(dm.w[0], n, nm.w[0], L)}};
-    cand = mask_rot<1>(cur, n - L, n, nm);  // bit p of cur -> bit (p + L) mod n
-  } else if (n_other <= kZnGapWalk) {
+  if (W == 1 && n_other * 2 <= n) {
+    cand.w[0] = zn_after_longest_runs(dm.w[0], n, nm.w[0], L);
+  } else if (W > 1 && n_other <= kZnGapWalk) {
     int first = -1, prev = -1;
 #pragma unroll
     for (int i = 0; i < W; ++i) {
