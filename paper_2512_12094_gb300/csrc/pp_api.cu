@@ -2,10 +2,11 @@
 //
 // A context owns two term tables of equal capacity (the live one and a
 // spare used as the destination of merges and compactions), a device
-// control block, and small constant tables.  By default all gates of a layer
-// run in one cooperative launch with a grid barrier between gates; otherwise
-// (and for batched rows) each gate is one kernel and repeated layers are
-// replayed from captured CUDA graphs.  The host reads the control block once
+// control block, and small constant tables.  By default a layer is applied as
+// phases over bucketed strings (apply_layer_phased); where those do not fit or
+// help, all its gates run in one cooperative launch with a grid barrier between
+// gates, or each gate is one kernel and repeated layers are replayed from
+// captured CUDA graphs.  The host reads the control block once
 // per layer: a gate that finds less than twice its input size free does
 // nothing and raises `stall`; the host then grows the tables and relaunches
 // the layer from that gate (earlier gates skip themselves).
@@ -510,9 +511,13 @@ pp_status make_room(pp_ctx* c, uint64_t factor = 2) {
   if (c->cfg.coeff_eps > 0.0 && c->n_terms > 0 && 4 * (c->n_terms - c->n_live) >= c->n_terms)
     PP_TRY(compact_into(c, 1 - c->active, 0.0, -1));
   const uint64_t cap = c->buf[c->active].cap;
-  if (factor * c->n_terms <= cap) return PP_OK;
-  const uint64_t least = c->n_terms * 4;
-  const uint64_t generous = std::max<uint64_t>(least, factor * c->n_terms * 3 / 2);
+  // no table needs more than twice the strings there are: a growth extrapolated
+  // from a first layer of a few terms is gigabytes otherwise, whose index every
+  // compaction clears (three layers on 8 qubits: 3 GB and 3.2 ms; so 10 MB and 3.0)
+  const uint64_t most = c->n <= 20 ? 2ull << (2 * c->n) : ~0ull;
+  if (std::min(factor * c->n_terms, most) <= cap) return PP_OK;
+  const uint64_t least = std::min(c->n_terms * 4, most);
+  const uint64_t generous = std::max<uint64_t>(least, std::min(factor * c->n_terms * 3 / 2, most));
   const pp_status st = ensure_capacity(c, generous);
   if (st != PP_ERR_CAPACITY || generous == least) return st;
   if (2 * c->n_terms <= cap) return PP_OK;  // the next gate fits; grow at a stall
