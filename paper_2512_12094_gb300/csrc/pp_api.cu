@@ -1283,7 +1283,7 @@ PhaseSizes phase_sizes(const pp_ctx* c, size_t G, size_t P) {
   z.cg = (256 + (uint64_t)(4.0 * z.est / (double)z.nb)) / 8 * 8;
   z.clear = sizeof(PhaseStat) + G * 24 + P * 8 + P * z.nb * 4;
   z.bytes = align256(z.clear) + align256(G * 4) +
-            2 * (align256(z.nb * z.cg * 8 * P32) + 2 * align256(z.nb * z.cg * 8));
+            2 * align256(z.nb * z.cg * phase_record_bytes(P32));
   if (c->batched) {
     // rows of the phases between, and of classes larger than shared memory
     const size_t row = (size_t)c->B * c->esize;
@@ -1365,12 +1365,8 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   {
     unsigned char* p = scratch + al(clear) + al(G * 4);
     for (int k = 0; k < 2; ++k) {
-      buckets[k].keys = reinterpret_cast<uint32_t*>(p);
-      p += al(nb * cg * 8 * P32);
-      buckets[k].coef = reinterpret_cast<double*>(p);
-      p += al(nb * cg * 8);
-      buckets[k].meta = reinterpret_cast<uint2*>(p);
-      p += al(nb * cg * 8);
+      buckets[k].rec = reinterpret_cast<uint4*>(p);
+      p += al(nb * cg * phase_record_bytes(P32));
       buckets[k].cnt = nullptr;
     }
     mid_rows = p;

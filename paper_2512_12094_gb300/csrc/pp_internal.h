@@ -226,14 +226,17 @@ struct PhaseDesc {
   uint64_t ux[kMaxW], uz[kMaxW];
 };
 
-// [nb][cg] entries, cnt[nb] appended so far (may pass cg: the bucket was full).
-// meta: gates of the phase active on the string, low half of its class hash.
+// [nb][cg] records, cnt[nb] appended so far (may pass cg: the bucket was full).
+// A record is 1 + (P + 1) / 2 units: coefficient, gates of the phase active on the
+// string and low half of its class hash; then the key, x words before z words.  Up
+// to 64 sites it is one 32-byte sector (in three arrays a string was three partial
+// ones: 20 merged layers of the 32-site ring 16.9 ms, 16.7 so; torus 5 x 6 35.8 and
+// 34.7).
 struct PhaseBuckets {
-  uint32_t* keys;  // [2 P] words a string: x words, then z words
-  double* coef;
-  uint2* meta;
+  uint4* rec;
   unsigned* cnt;
 };
+inline size_t phase_record_bytes(int P) { return (size_t)(1 + (P + 1) / 2) * 16; }
 
 struct PhaseRule {
   int use_eps;

@@ -391,9 +391,11 @@ __global__ void __launch_bounds__(kPT, kPBlocks)
       for (int u = 0; u < U; ++u) {
         const int i = i0 + 32 * u + lane;
         if (i < cnt) {
-          m[u] = in.meta[base + i];
-          K[u] = ld_pkey<P>(in.keys, base + i);
-          c[u] = in.coef[base + i];
+          const uint4* r = in.rec + (base + i) * kRecord<P>;
+          const uint4 a = r[0];
+          m[u] = make_uint2(a.z, a.w);
+          K[u] = ld_pkey<P>(reinterpret_cast<const uint32_t*>(r + 1), 0);
+          c[u] = __hiloint2double((int)a.y, (int)a.x);
         }
       }
 #pragma unroll
@@ -604,17 +606,18 @@ __global__ void __launch_bounds__(kDT, 2)
       __syncthreads();
       for (int i0 = 0; i0 < cnt; i0 += kDT) {
         const int i = i0 + tid;
-        uint2 m = make_uint2(0u, 0u);
-        if (i < cnt) m = in.meta[base + i];
-        const bool mine = i < cnt && (m.y & ((1u << s) - 1u)) == id;
+        const uint4* r = in.rec + (base + i) * kRecord<P>;
+        uint4 a = make_uint4(0u, 0u, 0u, 0u);
+        if (i < cnt) a = r[0];
+        const bool mine = i < cnt && (a.w & ((1u << s) - 1u)) == id;
         const unsigned bal = __ballot_sync(kFull, mine);
         int p = 0;
         if (lane == 0 && bal) p = atomicAdd(&S.n, __popc(bal));
         p = __shfl_sync(kFull, p, 0) + __popc(bal & below);
         if (mine && p < kDStrings) {
-          S.key[p] = pack_key<P>(ld_pkey<P>(in.keys, base + i));
-          S.coef[p] = in.coef[base + i];
-          S.act[p] = m.x;
+          S.key[p] = pack_key<P>(ld_pkey<P>(reinterpret_cast<const uint32_t*>(r + 1), 0));
+          S.coef[p] = __hiloint2double((int)a.y, (int)a.x);
+          S.act[p] = a.z;
         }
       }
       __syncthreads();

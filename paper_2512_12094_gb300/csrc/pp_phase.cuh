@@ -157,6 +157,9 @@ __device__ __forceinline__ void classify(const PKey<P>& K, const NextGens<P>& ne
   h = string_hash<P>(v, act);
 }
 
+template <int P>
+constexpr int kRecord = 1 + (P + 1) / 2;  // units of a bucket's record
+
 // Append a string to its bucket of the next phase.
 template <int P>
 __device__ __forceinline__ void deal(const PhaseBuckets& out, unsigned nb, unsigned cg,
@@ -166,9 +169,9 @@ __device__ __forceinline__ void deal(const PhaseBuckets& out, unsigned nb, unsig
   const unsigned p = atomicAdd(out.cnt + b, 1u);
   if (p < cg) {
     const uint64_t at = (uint64_t)b * cg + p;
-    st_pkey<P>(out.keys, at, K);
-    out.coef[at] = c;
-    out.meta[at] = make_uint2(act, (unsigned)h);
+    uint4* const r = out.rec + at * kRecord<P>;
+    r[0] = make_uint4((unsigned)__double2loint(c), (unsigned)__double2hiint(c), act, (unsigned)h);
+    st_pkey<P>(reinterpret_cast<uint32_t*>(r + 1), 0, K);
   } else {
     fail |= kPhaseBucketFull;
   }

@@ -142,13 +142,15 @@ __global__ void __launch_bounds__(256)
       if (tid == 0) S.n = S.classes = S.bad = 0;
       __syncthreads();
       for (int i = tid; i < cnt; i += NT) {
-        const uint2 m = in.meta[base + i];
+        const uint4* r = in.rec + (base + i) * kRecord<P>;
+        const uint4 head = r[0];
+        const uint2 m = make_uint2(head.z, head.w);
         if ((m.y & ((1u << s) - 1u)) != id) continue;
         const int p = atomicAdd(&S.n, 1);
         if (p >= kRStrings) continue;
-        S.row[p] = (uint32_t)__double_as_longlong(in.coef[base + i]);
+        S.row[p] = head.x;
         S.act[p] = m.x;
-        DKey<P> v = pack_key<P>(ld_pkey<P>(in.keys, base + i));
+        DKey<P> v = pack_key<P>(ld_pkey<P>(reinterpret_cast<const uint32_t*>(r + 1), 0));
         unsigned f = 0;
         if (__popc(m.x) > kDRank) {
           S.bad = 1;
