@@ -439,7 +439,8 @@ def bench_ours(args):
                      "traffic_basis": "ncu DRAM bytes per algorithmic byte of the last layer "
                                       "of the Z_32 job x this run's average launch; null when "
                                       "the kernel sources differ from the captured ones",
-                     "kernel": "layer_kernel<1>", "block_threads": stats[-1]["block_threads"],
+                     "kernel": "layers as phases (dense_phase_kernel<1>) and layer_kernel<1>",
+                     "block_threads": stats[-1]["block_threads"],
                      "peak_kind": peak_kind,
                      "peak_nominal": HBM_NOMINAL_GBS,
                      "frac_nominal": (achieved / HBM_NOMINAL_GBS) if achieved else None,

@@ -116,19 +116,23 @@ typedef struct {
   int profile_kernels;     /* nonzero: bracket every kernel that applies gates with CUDA
                               events on the context's stream and accumulate their
                               durations into pp_stats_t.gate_kernel_ms */
-  int layer_kernel;        /* nonzero (default): all gates of a layer run in one persistent
+  int layer_kernel;        /* nonzero (default): a layer is applied as phases, runs of gates
+                              over buckets of strings that never meet, or, where those do
+                              not fit or help, all its gates run in one persistent
                               cooperative kernel with a grid barrier between gates; zero:
                               one kernel per gate, replayed from CUDA graphs */
   int merge_method;        /* pp_merge_method of the symmetry and identical-string merges
                               after ingest (ingest itself uses the hash table) */
   int block_threads;       /* threads per block of the persistent layer kernel: 256 (several
                               blocks per SM) or 1024 (one per SM; one-word and two-word
-                              strings, single column); 0 = 256 */
+                              strings, single column); 0 = 256.  Layers of a context that
+                              sets it are not applied as phases */
   int wait_limit;          /* microseconds a bounded device wait (the grid barrier between
                               gates, a merge waiting for a claimed index slot) may last before
                               it gives up: the kernel records the failure and returns, and the
                               call reports PP_ERR_TIMEOUT; 0 = the default, 30 s (a gate over
-                              gigabytes of batched rows takes seconds).  >= 0. */
+                              gigabytes of batched rows takes seconds).  >= 0.  Layers of a
+                              context that sets it are not applied as phases */
   double room_factor;      /* headroom a layer asks for before its first gate: room for
                               2 x room_factor x (the previous layer's growth) times the
                               stored terms, and at least twice them; a layer that outgrows
@@ -148,7 +152,9 @@ typedef struct {
   int64_t merges;          /* symmetry or identical-string merges performed */
   int64_t compactions;
   int64_t regrows;
-  size_t device_bytes;     /* device memory currently held by the context */
+  size_t device_bytes;     /* device memory currently held by the context (a call's own
+                              scratch, such as the buckets of a layer's phases, is given
+                              back before it returns) */
   double anticommuting_terms; /* sum over applied gates of live terms anticommuting with P */
   int64_t kernel_launches; /* kernels launched by the context (graph nodes included) */
   double gate_kernel_ms;   /* with profile_kernels: summed duration of the kernels that applied
