@@ -22,6 +22,7 @@
 #include <algorithm>
 
 #include "pp_device.cuh"
+#include "pp_smem_limit.h"
 
 namespace cg = cooperative_groups;
 
@@ -962,9 +963,8 @@ __global__ void __launch_bounds__(kOvThreads)
 template <int W>
 cudaError_t launch_overlap_blocks(int grid, cudaStream_t s, const uint64_t* keys, const double* coef,
                                   uint64_t count, const OverlapArgs& a, double* partials) {
-  const cudaError_t e = cudaFuncSetAttribute(overlap_zn_blocks_kernel<W>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)overlap_blocks_smem(kOvSites));
+  static SmemLimit limit;
+  const cudaError_t e = limit.raise(overlap_zn_blocks_kernel<W>, overlap_blocks_smem(kOvSites));
   if (e != cudaSuccess) return e;
   overlap_zn_blocks_kernel<W><<<grid, kOvThreads, overlap_blocks_smem(a.n), s>>>(keys, coef, count, a,
                                                                                  partials);
@@ -1089,14 +1089,12 @@ cudaError_t launch_gate_w(int grid, cudaStream_t s, const DevTable* tab, DevCtl*
   return cudaLaunchKernelEx(&cfg, gate_kernel<W>, tab, ctl, g);
 }
 
-// The layer kernel's dynamic shared memory must be allowed above 48 KB once
-// per instantiation (and before an occupancy query).
+// The layer kernel's dynamic shared memory must be allowed above 48 KB before
+// a launch and before an occupancy query.
 template <int W, int NT>
 cudaError_t layer_smem_setup() {
-  static cudaError_t done = cudaFuncSetAttribute(
-      layer_kernel<W, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-      (int)sizeof(LayerSmem<W, NT>));
-  return done;
+  static SmemLimit limit;
+  return limit.raise(layer_kernel<W, NT>, sizeof(LayerSmem<W, NT>));
 }
 
 template <int W, int NT>

@@ -19,6 +19,7 @@
 #include <algorithm>
 
 #include "pp_phase.cuh"
+#include "pp_smem_limit.h"
 
 namespace ppk {
 namespace {
@@ -255,9 +256,8 @@ cudaError_t merge_pg(const MergeBuckets& m, cudaStream_t s, const DevTable& src,
                                                                           (uint64_t)sms * 8)),
                             kBlock, 0, s>>>(src.keys, src.coef, count, count_dev, skip_zero, n, lx,
                                             m, ctl, guarded);
-  static const cudaError_t e =
-      cudaFuncSetAttribute(merge_bucket_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)sizeof(MergeSmem<P>));
+  static SmemLimit limit;
+  const cudaError_t e = limit.raise(merge_bucket_kernel<P>, sizeof(MergeSmem<P>));
   if (e != cudaSuccess) return e;
   const int per_sm = std::min<int>(8, (int)(226 * 1024 / (sizeof(MergeSmem<P>) + 1024)));
   merge_bucket_kernel<P><<<(int)std::min<uint64_t>(m.nb, (uint64_t)sms * per_sm), kMT,

@@ -27,6 +27,7 @@
 #include <algorithm>
 
 #include "pp_phase.cuh"
+#include "pp_smem_limit.h"
 
 namespace ppk {
 namespace {
@@ -933,10 +934,8 @@ cudaError_t phase_setup() {
   static_assert(PhaseDims<P>::C < (1 << kPosBits) && 4 * PhaseDims<P>::C <= 3 * PhaseDims<P>::kSlots,
                 "positions fit an index slot; an index is never full");
   static_assert(kPBlocks * (sizeof(PhaseSmem<P>) + 1024) <= 228 * 1024, "blocks per SM");
-  static cudaError_t done =
-      cudaFuncSetAttribute(phase_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)sizeof(PhaseSmem<P>));
-  return done;
+  static SmemLimit limit;
+  return limit.raise(phase_kernel<P>, sizeof(PhaseSmem<P>));
 }
 
 template <int P>
@@ -957,9 +956,8 @@ cudaError_t launch_dense_p(int warps, cudaStream_t s, const PhaseBuckets& in, co
                            const GateArgs* gates, const PhaseRule& rule, const DevTable& dense,
                            DevCtl* ctl, const PhaseAcc& acc) {
   static_assert(2 * (sizeof(DenseSmem<P>) + 1024) <= 228 * 1024, "blocks per SM");
-  static const cudaError_t e =
-      cudaFuncSetAttribute(dense_phase_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)sizeof(DenseSmem<P>));
+  static SmemLimit limit;
+  const cudaError_t e = limit.raise(dense_phase_kernel<P>, sizeof(DenseSmem<P>));
   if (e != cudaSuccess) return e;
   // two blocks of 8 warps per SM where phase_kernel has three of 4
   const int grid = std::max(1, warps / (kPW * kPBlocks) * 2);

@@ -17,6 +17,7 @@
 #include <algorithm>
 
 #include "pp_phase.cuh"
+#include "pp_smem_limit.h"
 
 namespace ppk {
 namespace {
@@ -375,8 +376,8 @@ cudaError_t launch_rows_pt(const RowsLaunch& L, cudaStream_t s, const PhaseBucke
                            const PhaseDesc& next, const GateArgs* gates, const PhaseRule& rule,
                            const void* src, void* dst, uint64_t dst_cap, unsigned long long* n_out,
                            void* spill, const DevTable& dense, DevCtl* ctl, const PhaseAcc& acc) {
-  static const cudaError_t e = cudaFuncSetAttribute(
-      rows_phase_kernel<P, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  static SmemLimit limit;
+  const cudaError_t e = limit.raise(rows_phase_kernel<P, T>, 227 * 1024);
   if (e != cudaSuccess) return e;
   rows_phase_kernel<P, T><<<L.grid, L.threads, L.smem, s>>>(
       in, out, nb, cg, d, next, gates, static_cast<const T*>(src), static_cast<T*>(dst), dst_cap, n_out,
