@@ -323,6 +323,19 @@ const char* pp_last_error(void);
  * injection fires once; n < 0 turns it off.  Never touches the GPU. */
 pp_status pp_debug_fail_alloc_after(int64_t n);
 
+/* The ways the context's layers went, for tests: results do not depend on
+ * them.  Written to out[0..PP_ROUTES). */
+enum {
+  PP_ROUTE_PHASED = 0,        /* layers applied as phases (see layer_kernel) */
+  PP_ROUTE_BUCKET_FULL = 1,   /* begun as phases and given up: a bucket was full, */
+  PP_ROUTE_CLASS_FULL = 2,    /* a class was larger than a phase holds, */
+  PP_ROUTE_TABLE_FULL = 3,    /* or the strings outgrew the table */
+  PP_ROUTE_MERGE_BUCKETS = 4, /* symmetry merges of phased layers by buckets */
+  PP_ROUTE_MERGE_FULL = 5,    /* of them, given up and done by the hash index */
+  PP_ROUTES = 6
+};
+pp_status pp_debug_layer_routes(const pp_ctx* ctx, int64_t* out);
+
 /* ------------------------------------------------------------------------
  * Stateless entry points on caller-owned device arrays.  Keys are device
  * arrays [m][2W] with the x words of a string followed by its z words.  All

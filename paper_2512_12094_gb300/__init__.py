@@ -163,6 +163,7 @@ _SIGS = {
     "pp_synchronize": [_vp],
     "pp_last_error": [],
     "pp_debug_fail_alloc_after": [ctypes.c_int64],
+    "pp_debug_layer_routes": [ctypes.c_void_p, _i64p],
     "pp_canonical_keys": [ctypes.c_int, ctypes.c_int, ctypes.c_int64, _vp, _vp, _vp],
     "pp_merge_terms": [ctypes.c_int, ctypes.c_int, ctypes.c_int64, _vp, _vp, _vp, _vp, _i64p, _vp],
     "pp_merge_terms_sorted": [ctypes.c_int, ctypes.c_int, ctypes.c_int64, _vp, _vp, _vp, _vp, _i64p,
@@ -365,6 +366,14 @@ def pp_last_error() -> str:
 def pp_debug_fail_alloc_after(n: int):
     """Make the allocation after the next n fail as out of memory (n < 0: off)."""
     _check(load().pp_debug_fail_alloc_after(int(n)))
+
+
+def pp_debug_layer_routes(ctx) -> dict:
+    """How the context's layers were applied and merged so far (include/pp.h)."""
+    names = ("phased", "bucket_full", "class_full", "table_full", "merge_buckets", "merge_full")
+    out = (ctypes.c_int64 * len(names))()
+    _check(load().pp_debug_layer_routes(ctx, out))
+    return dict(zip(names, out))
 
 
 def pp_canonical_keys(n_qubits: int, symmetry: int, m: int, keys_in, keys_out, stream=None):

@@ -185,6 +185,7 @@ struct pp_ctx {
   int phase_wait = 0;          // layers left before phases are tried again
   int phase_fails = 0;         // phased layers given up in a row
   int phase_gates = kPhaseGates;  // of a phase at most
+  int64_t routes[PP_ROUTES] = {};
   float* h_activity = nullptr; // pinned, kActivityMax gates
   void* sort_scratch = nullptr;  // scratch of the sort-based merge (merge_method 1)
   size_t sort_scratch_bytes = 0;
@@ -1468,7 +1469,10 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   release(PP_OK);
   if (st == PP_OK) st = check_device_error(c);
   if (st != PP_OK) return st;
+  if (by_buckets && (!c->h_ctl->stall || c->h_ctl->stall == kMergeFull)) c->routes[PP_ROUTE_MERGE_BUCKETS]++;
   if (c->h_ctl->stall == kMergeFull) {
+    c->routes[PP_ROUTE_PHASED]++;
+    c->routes[PP_ROUTE_MERGE_FULL]++;
     // the gates are done, in the other table; their merge is left to the index
     c->phase_fails = 0;
     c->last_growth = (double)c->h_ctl->after_terms / (double)T;
@@ -1482,6 +1486,9 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   if (const unsigned why = c->h_ctl->stall) {
     // given up: the input table is whole (its index may not be).  Next time
     // with finer phases or more buckets, and after ever longer waits.
+    c->routes[(why & kPhaseClassFull)    ? PP_ROUTE_CLASS_FULL
+              : (why & kPhaseBucketFull) ? PP_ROUTE_BUCKET_FULL
+                                         : PP_ROUTE_TABLE_FULL]++;
     if (why & kPhaseClassFull) {
       // a dense class of more active gates than its room (a star of bonds):
       // then no phase has more gates than that
@@ -1498,6 +1505,7 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
     return PP_OK;
   }
   c->phase_fails = 0;
+  c->routes[PP_ROUTE_PHASED]++;
   if (c->cfg.profile_kernels) {
     float ms = 0.f;
     PP_CUDA(cudaEventElapsedTime(&ms, c->ev_layer[0], c->ev_layer[1]));
@@ -1669,6 +1677,12 @@ pp_status pp_config_default(pp_config* cfg) {
 
 pp_status pp_debug_fail_alloc_after(int64_t n) {
   g_fail_alloc_after.store(n < 0 ? -1 : (long long)n);
+  return PP_OK;
+}
+
+pp_status pp_debug_layer_routes(const pp_ctx* c, int64_t* out) {
+  if (!c || !out) return fail(PP_ERR_ARG, "null argument");
+  std::copy(c->routes, c->routes + PP_ROUTES, out);
   return PP_OK;
 }
 

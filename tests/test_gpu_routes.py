@@ -1,0 +1,77 @@
+"""Which way a layer went: as phases, given up and applied by the persistent
+kernel, merged by buckets or by the index (pp_debug_layer_routes).  Every way gives
+the same table, so a comparison of tables does not show that one was taken (needs a
+GB300)."""
+import numpy as np
+import pytest
+
+import paper_2512_12094_gb300 as pp
+import pp_inputs as pi
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    pp.build()
+    pp.load()
+
+
+def routes_of(wl, symmetry, **kw):
+    """(routes, entries of the table)"""
+    p = pp.Propagator.from_workload(wl, symmetry=symmetry, **kw)
+    for layer in reversed(range(len(wl.circuit.layers))):
+        gx, gz, th = wl.circuit.gate_arrays(layer)
+        p.apply_layer(gx, gz, th, True)
+    r, n = pp.pp_debug_layer_routes(p.ctx), p.num_terms()[0]
+    p.close()
+    return r, n
+
+
+GIVEN_UP = ("bucket_full", "class_full", "table_full")
+
+
+@pytest.mark.parametrize("n,eps,wmax", [(32, 1e-4, 10), (64, 1e-4, 8), (40, 0.0, 4), (100, 1e-3, 6)])
+def test_ring_layers_are_phased(n, eps, wmax):
+    """Dense phases of one and two words, sparse ones with and without truncation."""
+    r, _ = routes_of(pi.config1_ring(n=n, steps=6, eps=eps, max_weight=wmax), 0)
+    assert r["phased"] == 6 and not any(r[k] for k in GIVEN_UP)
+
+
+@pytest.mark.parametrize("kw", [dict(block_threads=256), dict(wait_limit=10 ** 7), dict(layer_kernel=False),
+                                dict(budget=4 << 20)])
+def test_layers_that_are_not(kw):
+    """The settings that name the other kernels, and a budget without room for the
+    buckets: 304 buckets of 256 records of 32 bytes, twice, take 5 MB."""
+    wl = pi.config1_ring(n=32, steps=4, eps=1e-3, max_weight=10)
+    r, _ = routes_of(wl, 0, **kw)
+    assert not any(r.values())
+
+
+@pytest.mark.parametrize("group,n,by_buckets,least", [(1, 32, True, 6), (3, 24, True, 6), (2, 24, False, 1)])
+def test_merges_of_phased_layers(group, n, by_buckets, least):
+    if group == 2:
+        wl = pi.config2_all_to_all(n, 0.02, 3, 0.01, 1e-4, 1, 2)
+    else:
+        wl = pi.config1_ring(n=n, steps=11, eps=1e-4, max_weight=9)
+    r, _ = routes_of(wl, group)
+    assert r["phased"] >= least
+    assert (r["merge_buckets"] > 0) == by_buckets and r["merge_full"] == 0
+
+
+@pytest.mark.parametrize("B,f32", [(64, False), (100, True)])
+def test_batched_layers_are_phased(B, f32):
+    n = 24
+    angles = pi.batched_ring_angles(B, 1)
+    gx, gz, _ = pi.Circuit(n, [pi.ring_layer(n, 0.0, 0.0, 0.0)]).gate_arrays(0)
+    x, z, c = pi.mean_z(n).arrays()
+    p = pp.Propagator(n, x, z, np.repeat(c[:, None], B, axis=1), eps=1e-5, batch=B, f32=f32)
+    for _ in range(2):
+        p.apply_layer(gx, gz, np.repeat(angles.T, n, axis=0), True)
+    assert pp.pp_debug_layer_routes(p.ctx)["phased"] == 2
+    p.close()
+
+
+def test_a_full_table_is_counted():
+    r, _ = routes_of(pi.config1_ring(n=40, steps=5, eps=1e-5, max_weight=7), 0, room_factor=0.01)
+    assert r["table_full"] > 0
