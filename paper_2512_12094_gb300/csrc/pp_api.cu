@@ -1260,31 +1260,36 @@ constexpr size_t kPhaseBytesMax = (size_t)64 << 30;
 
 size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
-// Buckets of a phased layer of G gates in P phases, and its scratch.  One bucket
-// per resident warp (dense: block) at least, and enough that a bucket of the
-// expected table fills half a warp's room (dense: kDenseFill strings of the
-// block's 1024; 500 measured 1 to 6 % slower, 1200 the same).  A bucket has room
-// for four times that and more, since classes come in lumps.
+// Buckets of a phased layer of G gates, and its scratch.  One bucket per resident
+// warp (dense: block) at least, and enough that a bucket of the expected table fills
+// half a warp's room (dense: kDenseFill strings of the block's 1024; 500 measured 1
+// to 6 % slower, 1200 the same).
 struct PhaseSizes {
   double est;  // strings expected at the layer's end
-  uint64_t nb, cg;
+  std::vector<ppphase::Room> rooms;  // of each phase
+  size_t counters, records;          // bytes of all phases' counters, and of the largest phase's records
   size_t clear, bytes, rows = 0, spill = 0;
+  uint64_t most;                     // buckets of a phase
 };
 
-PhaseSizes phase_sizes(const pp_ctx* c, size_t G, size_t P) {
+PhaseSizes phase_sizes(const pp_ctx* c, size_t G, const std::vector<ppphase::Phase>& phases) {
   PhaseSizes z;
   const int P32 = phase_words(c->n);
-  const bool dense = dense_classes(c);
+  const size_t P = phases.size();
   z.est = (double)c->n_terms * std::max(1.5, 1.25 * c->last_growth);
-  const double half = c->batched ? kRowsFill
-                      : dense    ? kDenseFill
-                                 : 0.5 * phase_strings_per_warp(P32);
-  const uint64_t least = (uint64_t)c->sms * (c->batched ? 8 : dense ? 2 : phase_warps_per_sm());
-  z.nb = std::max<uint64_t>(least, (uint64_t)std::ceil(z.est * c->phase_room / half));
-  z.cg = (256 + (uint64_t)(4.0 * z.est / (double)z.nb)) / 8 * 8;
-  z.clear = sizeof(PhaseStat) + G * 24 + P * 8 + P * z.nb * 4;
-  z.bytes = align256(z.clear) + align256(G * 4) +
-            2 * align256(z.nb * z.cg * phase_record_bytes(P32));
+  const ppphase::Workers warps = {0.5 * phase_strings_per_warp(P32), (uint64_t)c->sms * phase_warps_per_sm()};
+  const ppphase::Workers blocks = c->batched ? ppphase::Workers{kRowsFill, (uint64_t)c->sms * 8}
+                                             : ppphase::Workers{kDenseFill, (uint64_t)c->sms * 2};
+  z.rooms = ppphase::bucket_rooms(phases, z.est, blocks, warps, c->phase_room);
+  z.counters = z.records = 0;
+  z.most = 0;
+  for (const ppphase::Room& r : z.rooms) {
+    z.counters += r.nb * 4;
+    z.records = std::max(z.records, align256(r.nb * r.cg * phase_record_bytes(P32)));
+    z.most = std::max(z.most, r.nb);
+  }
+  z.clear = sizeof(PhaseStat) + G * 24 + P * 8 + z.counters;
+  z.bytes = align256(z.clear) + align256(G * 4) + 2 * z.records;
   if (c->batched) {
     // rows of the phases between, and of classes larger than shared memory
     const size_t row = (size_t)c->B * c->esize;
@@ -1330,8 +1335,7 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
     for (const ppphase::Phase& ph : phases)
       if (!ph.triangular) return PP_OK;
   Range range_("phases");
-  const PhaseSizes z = phase_sizes(c, G, P);
-  const uint64_t nb = z.nb, cg = z.cg;
+  const PhaseSizes z = phase_sizes(c, G, phases);
   const size_t need = z.bytes;
   const double est = z.est;
   const int P32 = phase_words(c->n);
@@ -1341,7 +1345,7 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   const int warps = c->sms * phase_warps_per_sm();
   auto al = align256;
   const size_t clear = z.clear;
-  if (nb >= (1ull << 26) || need > kPhaseBytesMax) return PP_OK;
+  if (z.most >= (1ull << 26) || need > kPhaseBytesMax) return PP_OK;
   if (c->cfg.mem_budget_bytes && c->bytes + need > c->cfg.mem_budget_bytes) return PP_OK;
   unsigned char* scratch = nullptr;
   if (dmalloc(c, (void**)&scratch, need) != PP_OK) {  // no room for it: the other path
@@ -1367,12 +1371,20 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
     unsigned char* p = scratch + al(clear) + al(G * 4);
     for (int k = 0; k < 2; ++k) {
       buckets[k].rec = reinterpret_cast<uint4*>(p);
-      p += al(nb * cg * phase_record_bytes(P32));
-      buckets[k].cnt = nullptr;
+      p += z.records;
     }
     mid_rows = p;
     spill = p + z.rows;
   }
+  std::vector<unsigned*> counters(1, cnt);  // of each phase's buckets
+  for (const ppphase::Room& r : z.rooms) counters.push_back(counters.back() + r.nb);
+  auto buckets_of = [&](size_t p) {
+    PhaseBuckets b = buckets[p & 1];
+    b.cnt = p < P ? counters[p] : nullptr;
+    b.nb = p < P ? (unsigned)z.rooms[p].nb : 0u;
+    b.cg = p < P ? (unsigned)z.rooms[p].cg : 0u;
+    return b;
+  };
   std::vector<int> skip_after(G + 1, 0);  // gates from g on that touch nothing
   for (size_t g = G; g-- > 0;) skip_after[g] = skip_after[g + 1] + !touch[g];
   auto desc = [&](size_t p) {
@@ -1403,36 +1415,28 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   auto run = [&](cudaError_t r) { e = (e == cudaSuccess) ? r : e; };
   if (c->cfg.profile_kernels) run(cudaEventRecord(c->ev_layer[0], c->stream));
   run(launch_phase_begin(c->stream, acc, clear, c->d_ctl, c->sms));
-  buckets[0].cnt = cnt;
   const int dgrid = (int)std::min<uint64_t>((T + kBlock - 1) / kBlock, (uint64_t)c->sms * 8);
   if (c->batched) {
     const RowsLaunch L = rows_launch(P32, c->B, (int)c->esize, c->sms);
-    run(launch_rows_deal(P32, dgrid, c->stream, desc_of(c, c->buf[src]), T, buckets[0], (unsigned)nb,
-                         (unsigned)cg, desc(0), ent.d_args, acc));
+    run(launch_rows_deal(P32, dgrid, c->stream, desc_of(c, c->buf[src]), T, buckets_of(0),
+                         desc(0), ent.d_args, acc));
     const void* from = c->buf[src].rows;
     for (size_t p = 0; p < P; ++p) {
-      PhaseBuckets in = buckets[p & 1], out = buckets[(p + 1) & 1];
-      in.cnt = cnt + p * nb;
-      out.cnt = p + 1 < P ? cnt + (p + 1) * nb : nullptr;
       // the last phase writes the destination table's rows, those before it
       // take turns with the rows between; the source's stay whole
       void* to = (P - 1 - p) % 2 == 0 ? c->buf[dst].rows : (void*)mid_rows;
-      run(launch_rows_phase(P32, L, c->stream, in, out, (unsigned)nb, (unsigned)cg, desc(p), desc(p + 1),
+      run(launch_rows_phase(P32, L, c->stream, buckets_of(p), buckets_of(p + 1), desc(p), desc(p + 1),
                             ent.d_args, rule, from, to, c->buf[dst].cap,
                             p + 1 < P ? written + p : &c->d_ctl->n_next, spill,
                             desc_of(c, c->buf[dst]), c->d_ctl, acc));
       from = to;
     }
   } else {
-    run(launch_phase_deal(P32, dgrid, c->stream, desc_of(c, c->buf[src]), T, rule.use_eps, buckets[0],
-                          (unsigned)nb, (unsigned)cg, desc(0), ent.d_args, acc));
-    for (size_t p = 0; p < P; ++p) {
-      PhaseBuckets in = buckets[p & 1], out = buckets[(p + 1) & 1];
-      in.cnt = cnt + p * nb;
-      out.cnt = p + 1 < P ? cnt + (p + 1) * nb : nullptr;
-      run(launch_phase(P32, warps, c->stream, in, out, (unsigned)nb, (unsigned)cg, desc(p), desc(p + 1),
+    run(launch_phase_deal(P32, dgrid, c->stream, desc_of(c, c->buf[src]), T, rule.use_eps, buckets_of(0),
+                          desc(0), ent.d_args, acc));
+    for (size_t p = 0; p < P; ++p)
+      run(launch_phase(P32, warps, c->stream, buckets_of(p), buckets_of(p + 1), desc(p), desc(p + 1),
                        ent.d_args, rule, desc_of(c, c->buf[dst]), c->d_ctl, acc));
-    }
   }
   run(launch_phase_end(c->stream, c->d_ctl, acc, (unsigned)G));
   if (c->cfg.profile_kernels) run(cudaEventRecord(c->ev_layer[1], c->stream));
@@ -2450,6 +2454,8 @@ size_t ppk::layer_scratch_bytes(const pp_ctx* c, int n_gates) {
   if (!c || c->batched || !c->cfg.layer_kernel || c->layer_bps <= 0 || !phases_allowed(c) ||
       n_gates < kPhaseMinGates)
     return 0;
-  const size_t bytes = phase_sizes(c, (size_t)n_gates, kPhaseMax).bytes;
+  ppphase::Phase kind;
+  kind.triangular = dense_classes(c);
+  const size_t bytes = phase_sizes(c, (size_t)n_gates, std::vector<ppphase::Phase>(kPhaseMax, kind)).bytes;
   return bytes > kPhaseBytesMax ? 0 : bytes;
 }

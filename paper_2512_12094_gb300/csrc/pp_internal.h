@@ -226,7 +226,8 @@ struct PhaseDesc {
   uint64_t ux[kMaxW], uz[kMaxW];
 };
 
-// [nb][cg] records, cnt[nb] appended so far (may pass cg: the bucket was full).
+// Buckets of one phase: [nb][cg] records, cnt[nb] appended so far (may pass cg: the
+// bucket was full).
 // A record is 1 + (P + 1) / 2 units: coefficient, gates of the phase active on the
 // string and low half of its class hash; then the key, x words before z words.  Up
 // to 64 sites it is one 32-byte sector (in three arrays a string was three partial
@@ -235,6 +236,7 @@ struct PhaseDesc {
 struct PhaseBuckets {
   uint4* rec;
   unsigned* cnt;
+  unsigned nb, cg;
 };
 inline size_t phase_record_bytes(int P) { return (size_t)(1 + (P + 1) / 2) * 16; }
 
@@ -283,12 +285,12 @@ cudaError_t launch_phase_begin(cudaStream_t s, const PhaseAcc& acc, size_t clear
                                int sms);
 // Live entries of src[0, T) into the buckets of phase d.
 cudaError_t launch_phase_deal(int P, int grid, cudaStream_t s, const DevTable& src, uint64_t T,
-                              int use_eps, const PhaseBuckets& out, unsigned nb, unsigned cg,
-                              const PhaseDesc& d, const GateArgs* gates, const PhaseAcc& acc);
+                              int use_eps, const PhaseBuckets& out, const PhaseDesc& d,
+                              const GateArgs* gates, const PhaseAcc& acc);
 // Phase d from `in`, on `warps` warps; survivors into `out` (the buckets of `next`) or, when
 // next.count is 0, appended to dense at ctl->n_next.
 cudaError_t launch_phase(int P, int warps, cudaStream_t s, const PhaseBuckets& in,
-                         const PhaseBuckets& out, unsigned nb, unsigned cg, const PhaseDesc& d,
+                         const PhaseBuckets& out, const PhaseDesc& d,
                          const PhaseDesc& next, const GateArgs* gates, const PhaseRule& rule,
                          const DevTable& dense, DevCtl* ctl, const PhaseAcc& acc);
 // Merge by buckets (pp_merge.cu), any group but S_n (whose orbits may all be one):
@@ -320,12 +322,12 @@ struct RowsLaunch {
 };
 RowsLaunch rows_launch(int P, int B, int esize, int sms);
 cudaError_t launch_rows_deal(int P, int grid, cudaStream_t s, const DevTable& src, uint64_t T,
-                             const PhaseBuckets& out, unsigned nb, unsigned cg, const PhaseDesc& d,
+                             const PhaseBuckets& out, const PhaseDesc& d,
                              const GateArgs* gates, const PhaseAcc& acc);
 // Phase d: rows src -> dst (room for dst_cap, *n_out written so far); after the
 // last phase keys and liveness of `dense` too, whose B and f32 describe the rows.
 cudaError_t launch_rows_phase(int P, const RowsLaunch& L, cudaStream_t s, const PhaseBuckets& in,
-                              const PhaseBuckets& out, unsigned nb, unsigned cg, const PhaseDesc& d,
+                              const PhaseBuckets& out, const PhaseDesc& d,
                               const PhaseDesc& next, const GateArgs* gates, const PhaseRule& rule,
                               const void* src, void* dst, uint64_t dst_cap, unsigned long long* n_out,
                               void* spill, const DevTable& dense, DevCtl* ctl, const PhaseAcc& acc);

@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(kBlock)
 template <int P>
 __global__ void __launch_bounds__(kBlock)
     phase_deal_kernel(const uint64_t* __restrict__ keys, const double* __restrict__ coef, uint64_t T,
-                      int use_eps, PhaseBuckets out, unsigned nb, unsigned cg, PhaseDesc d,
+                      int use_eps, PhaseBuckets out, PhaseDesc d,
                       const GateArgs* __restrict__ gates, PhaseAcc acc) {
   __shared__ __align__(16) NextGens<P> next;
   __shared__ unsigned s_live;
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(kBlock)
     unsigned act;
     uint64_t h;
     classify<P>(K, next, d, act, h);
-    deal<P>(out, nb, cg, K, c, act, h, fail);
+    deal<P>(out, K, c, act, h, fail);
   }
   live = __reduce_add_sync(kFull, live);
   if ((threadIdx.x & 31) == 0) atomicAdd(&s_live, live);
@@ -319,7 +319,7 @@ __device__ __forceinline__ int phase_gates(PhaseWarp<P>& S, const PGate<P>* gate
 // the dense table `dense`.
 template <int P>
 __global__ void __launch_bounds__(kPT, kPBlocks)
-    phase_kernel(PhaseBuckets in, PhaseBuckets out, unsigned nb, unsigned cg, PhaseDesc d,
+    phase_kernel(PhaseBuckets in, PhaseBuckets out, PhaseDesc d,
                  PhaseDesc next, const GateArgs* __restrict__ gates, PhaseRule rule, DevTable dense,
                  DevCtl* ctl, PhaseAcc acc) {
   extern __shared__ __align__(16) unsigned char phase_raw[];
@@ -365,11 +365,11 @@ __global__ void __launch_bounds__(kPT, kPBlocks)
   uint64_t base = 0;
   auto open = [&]() {  // the next bucket that holds anything
     cnt = 0;
-    for (; b < nb; b += warps) {
-      cnt = (int)min(in.cnt[b], cg);
+    for (; b < in.nb; b += warps) {
+      cnt = (int)min(in.cnt[b], in.cg);
       if (cnt) break;
     }
-    base = (uint64_t)b * cg;
+    base = (uint64_t)b * in.cg;
     s0 = 0;
     while ((cnt >> s0) > C * 3 / 4) ++s0;
     s = s0;
@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(kPT, kPBlocks)
         unsigned act;
         uint64_t h;
         classify<P>(K, B.next, next, act, h);
-        deal<P>(out, nb, cg, K, c, act, h, fail);
+        deal<P>(out, K, c, act, h, fail);
       }
     } else {
       // one reservation per part
@@ -555,7 +555,7 @@ struct DenseSmem {
 
 template <int P>
 __global__ void __launch_bounds__(kDT, 2)
-    dense_phase_kernel(PhaseBuckets in, PhaseBuckets out, unsigned nb, unsigned cg, PhaseDesc d,
+    dense_phase_kernel(PhaseBuckets in, PhaseBuckets out, PhaseDesc d,
                        PhaseDesc next, const GateArgs* __restrict__ gates, PhaseRule rule,
                        DevTable dense, DevCtl* ctl, PhaseAcc acc) {
   extern __shared__ __align__(16) unsigned char phase_raw[];
@@ -587,10 +587,10 @@ __global__ void __launch_bounds__(kDT, 2)
   long long upd = 0, skipped = 0;
   unsigned long long n_ac = 0;
   OccAcc<1> occ;
-  for (unsigned b = blockIdx.x; b < nb; b += gridDim.x) {
-    const int cnt = (int)min(in.cnt[b], cg);
+  for (unsigned b = blockIdx.x; b < in.nb; b += gridDim.x) {
+    const int cnt = (int)min(in.cnt[b], in.cg);
     if (cnt == 0) continue;
-    const uint64_t base = (uint64_t)b * cg;
+    const uint64_t base = (uint64_t)b * in.cg;
     // parts of the bucket, as in phase_kernel
     int s0 = 0;
     while ((cnt >> s0) > kDStrings * 3 / 4) ++s0;
@@ -815,7 +815,7 @@ __global__ void __launch_bounds__(kDT, 2)
           unsigned act;
           uint64_t h;
           classify<P>(K, S.next, next, act, h);
-          deal<P>(out, nb, cg, K, S.slot[k], act, h, fail);
+          deal<P>(out, K, S.slot[k], act, h, fail);
         }
       } else {
         if (tid == 0) S.out_base = atomicAdd(&ctl->n_next, (unsigned long long)n_live);
@@ -940,19 +940,19 @@ cudaError_t phase_setup() {
 
 template <int P>
 cudaError_t launch_phase_pt(int warps, cudaStream_t s, const PhaseBuckets& in, const PhaseBuckets& out,
-                            unsigned nb, unsigned cg, const PhaseDesc& d, const PhaseDesc& next,
+                            const PhaseDesc& d, const PhaseDesc& next,
                             const GateArgs* gates, const PhaseRule& rule, const DevTable& dense,
                             DevCtl* ctl, const PhaseAcc& acc) {
   const cudaError_t e = phase_setup<P>();
   if (e != cudaSuccess) return e;
   phase_kernel<P><<<std::max(1, warps / kPW), kPT, sizeof(PhaseSmem<P>), s>>>(
-      in, out, nb, cg, d, next, gates, rule, dense, ctl, acc);
+      in, out, d, next, gates, rule, dense, ctl, acc);
   return cudaGetLastError();
 }
 
 template <int P>
 cudaError_t launch_dense_p(int warps, cudaStream_t s, const PhaseBuckets& in, const PhaseBuckets& out,
-                           unsigned nb, unsigned cg, const PhaseDesc& d, const PhaseDesc& next,
+                           const PhaseDesc& d, const PhaseDesc& next,
                            const GateArgs* gates, const PhaseRule& rule, const DevTable& dense,
                            DevCtl* ctl, const PhaseAcc& acc) {
   static_assert(2 * (sizeof(DenseSmem<P>) + 1024) <= 228 * 1024, "blocks per SM");
@@ -961,7 +961,7 @@ cudaError_t launch_dense_p(int warps, cudaStream_t s, const PhaseBuckets& in, co
   if (e != cudaSuccess) return e;
   // two blocks of 8 warps per SM where phase_kernel has three of 4
   const int grid = std::max(1, warps / (kPW * kPBlocks) * 2);
-  dense_phase_kernel<P><<<grid, kDT, sizeof(DenseSmem<P>), s>>>(in, out, nb, cg, d, next, gates, rule,
+  dense_phase_kernel<P><<<grid, kDT, sizeof(DenseSmem<P>), s>>>(in, out, d, next, gates, rule,
                                                                 dense, ctl, acc);
   return cudaGetLastError();
 }
@@ -1002,22 +1002,22 @@ cudaError_t launch_phase_begin(cudaStream_t s, const PhaseAcc& acc, size_t clear
   }
 
 cudaError_t launch_phase_deal(int P, int grid, cudaStream_t s, const DevTable& src, uint64_t T,
-                              int use_eps, const PhaseBuckets& out, unsigned nb, unsigned cg,
-                              const PhaseDesc& d, const GateArgs* gates, const PhaseAcc& acc) {
-  PPP_DISPATCH(P, (phase_deal_kernel<PP><<<grid, kBlock, 0, s>>>(src.keys, src.coef, T, use_eps, out,
-                                                                 nb, cg, d, gates, acc)));
+                              int use_eps, const PhaseBuckets& out, const PhaseDesc& d,
+                              const GateArgs* gates, const PhaseAcc& acc) {
+  PPP_DISPATCH(P, (phase_deal_kernel<PP><<<grid, kBlock, 0, s>>>(src.keys, src.coef, T, use_eps, out, d,
+                                                                 gates, acc)));
   return cudaGetLastError();
 }
 
 cudaError_t launch_phase(int P, int warps, cudaStream_t s, const PhaseBuckets& in,
-                         const PhaseBuckets& out, unsigned nb, unsigned cg, const PhaseDesc& d,
+                         const PhaseBuckets& out, const PhaseDesc& d,
                          const PhaseDesc& next, const GateArgs* gates, const PhaseRule& rule,
                          const DevTable& dense, DevCtl* ctl, const PhaseAcc& acc) {
   if (d.dense && P <= 2) {
-    if (P == 1) return launch_dense_p<1>(warps, s, in, out, nb, cg, d, next, gates, rule, dense, ctl, acc);
-    return launch_dense_p<2>(warps, s, in, out, nb, cg, d, next, gates, rule, dense, ctl, acc);
+    if (P == 1) return launch_dense_p<1>(warps, s, in, out, d, next, gates, rule, dense, ctl, acc);
+    return launch_dense_p<2>(warps, s, in, out, d, next, gates, rule, dense, ctl, acc);
   }
-  PPP_DISPATCH(P, return (launch_phase_pt<PP>(warps, s, in, out, nb, cg, d, next, gates, rule, dense,
+  PPP_DISPATCH(P, return (launch_phase_pt<PP>(warps, s, in, out, d, next, gates, rule, dense,
                                               ctl, acc)));
   return cudaErrorInvalidValue;
 }

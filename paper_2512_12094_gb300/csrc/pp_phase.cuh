@@ -162,13 +162,12 @@ constexpr int kRecord = 1 + (P + 1) / 2;  // units of a bucket's record
 
 // Append a string to its bucket of the next phase.
 template <int P>
-__device__ __forceinline__ void deal(const PhaseBuckets& out, unsigned nb, unsigned cg,
-                                     const PKey<P>& K, double c, unsigned act, uint64_t h,
-                                     unsigned& fail) {
-  const unsigned b = (unsigned)(((h >> 32) * (uint64_t)nb) >> 32);
+__device__ __forceinline__ void deal(const PhaseBuckets& out, const PKey<P>& K, double c, unsigned act,
+                                     uint64_t h, unsigned& fail) {
+  const unsigned b = (unsigned)(((h >> 32) * (uint64_t)out.nb) >> 32);
   const unsigned p = atomicAdd(out.cnt + b, 1u);
-  if (p < cg) {
-    const uint64_t at = (uint64_t)b * cg + p;
+  if (p < out.cg) {
+    const uint64_t at = (uint64_t)b * out.cg + p;
     uint4* const r = out.rec + at * kRecord<P>;
     r[0] = make_uint4((unsigned)__double2loint(c), (unsigned)__double2hiint(c), act, (unsigned)h);
     st_pkey<P>(reinterpret_cast<uint32_t*>(r + 1), 0, K);

@@ -175,4 +175,36 @@ inline std::vector<Phase> plan(const std::vector<Gen>& gates, int W, const unsig
   return out;
 }
 
+// Buckets of one phase, and the records each has room for.
+struct Room {
+  uint64_t nb = 0, cg = 0;
+};
+
+// What takes a phase's buckets, a block or a warp each: how many strings one is to
+// hold, and how many buckets keep the chip busy.
+struct Workers {
+  double fill;
+  uint64_t least;
+};
+
+// For `strings` expected at the layer's end.  A bucket has room for four times its
+// share and more, since classes come in lumps.
+inline Room bucket_room(double strings, const Workers& w, double factor) {
+  Room r;
+  const uint64_t n = (uint64_t)std::ceil(strings * factor / w.fill);
+  r.nb = n > w.least ? n : w.least;
+  r.cg = (256 + (uint64_t)(4.0 * strings / (double)r.nb)) / 8 * 8;
+  return r;
+}
+
+// Each phase's, by what takes its buckets.  (With the buckets of the blocks for all,
+// all-to-all layers with truncation, whose phases are not dense, ran on 304 of 1824
+// warps; with those of the warps for all, a dense phase takes many times the parts.)
+inline std::vector<Room> bucket_rooms(const std::vector<Phase>& phases, double strings, const Workers& dense,
+                                      const Workers& sparse, double factor) {
+  std::vector<Room> out;
+  for (const Phase& p : phases) out.push_back(bucket_room(strings, p.triangular ? dense : sparse, factor));
+  return out;
+}
+
 }  // namespace ppphase

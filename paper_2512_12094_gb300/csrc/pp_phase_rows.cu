@@ -70,7 +70,7 @@ struct RowsSmem {
 template <int P>
 __global__ void __launch_bounds__(kBlock)
     rows_deal_kernel(const uint64_t* __restrict__ keys, const unsigned char* __restrict__ alive,
-                     uint64_t T, PhaseBuckets out, unsigned nb, unsigned cg, PhaseDesc d,
+                     uint64_t T, PhaseBuckets out, PhaseDesc d,
                      const GateArgs* __restrict__ gates, PhaseAcc acc) {
   __shared__ __align__(16) NextGens<P> next;
   __shared__ unsigned s_live;
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kBlock)
     unsigned act;
     uint64_t h;
     classify<P>(K, next, d, act, h);
-    deal<P>(out, nb, cg, K, __longlong_as_double((long long)i), act, h, fail);
+    deal<P>(out, K, __longlong_as_double((long long)i), act, h, fail);
   }
   live = __reduce_add_sync(kFull, live);
   if ((threadIdx.x & 31) == 0) atomicAdd(&s_live, live);
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kBlock)
 // next.count == 0 the keys and liveness of `dense` are written too.
 template <int P, typename T>
 __global__ void __launch_bounds__(256)
-    rows_phase_kernel(PhaseBuckets in, PhaseBuckets out, unsigned nb, unsigned cg, PhaseDesc d,
+    rows_phase_kernel(PhaseBuckets in, PhaseBuckets out, PhaseDesc d,
                       PhaseDesc next, const GateArgs* __restrict__ gates, const T* __restrict__ src,
                       T* dst, uint64_t dst_cap, unsigned long long* n_out, int B, int use_eps,
                       double eps, int wmax, int smem_rows, T* spill, DevTable dense, DevCtl* ctl,
@@ -128,10 +128,10 @@ __global__ void __launch_bounds__(256)
   long long upd = 0, skipped = 0;  // of thread 0
   unsigned long long n_ac = 0;
   OccAcc<1> occ;
-  for (unsigned b = blockIdx.x; b < nb; b += gridDim.x) {
-    const int cnt = (int)min(in.cnt[b], cg);
+  for (unsigned b = blockIdx.x; b < in.nb; b += gridDim.x) {
+    const int cnt = (int)min(in.cnt[b], in.cg);
     if (cnt == 0) continue;
-    const uint64_t base = (uint64_t)b * cg;
+    const uint64_t base = (uint64_t)b * in.cg;
     int s0 = 0;
     while ((cnt >> s0) > kRStrings * 3 / 4) ++s0;
     int s = s0;
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(256)
               unsigned na;
               uint64_t h;
               classify<P>(K, S.next, next, na, h);
-              deal<P>(out, nb, cg, K, __longlong_as_double((long long)at), na, h, fail);
+              deal<P>(out, K, __longlong_as_double((long long)at), na, h, fail);
             } else {
               Key<1> K;
               K.x(0) = x_of<P>(w);
@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(256)
 
 template <int P, typename T>
 cudaError_t launch_rows_pt(const RowsLaunch& L, cudaStream_t s, const PhaseBuckets& in,
-                           const PhaseBuckets& out, unsigned nb, unsigned cg, const PhaseDesc& d,
+                           const PhaseBuckets& out, const PhaseDesc& d,
                            const PhaseDesc& next, const GateArgs* gates, const PhaseRule& rule,
                            const void* src, void* dst, uint64_t dst_cap, unsigned long long* n_out,
                            void* spill, const DevTable& dense, DevCtl* ctl, const PhaseAcc& acc) {
@@ -380,7 +380,7 @@ cudaError_t launch_rows_pt(const RowsLaunch& L, cudaStream_t s, const PhaseBucke
   const cudaError_t e = limit.raise(rows_phase_kernel<P, T>, 227 * 1024);
   if (e != cudaSuccess) return e;
   rows_phase_kernel<P, T><<<L.grid, L.threads, L.smem, s>>>(
-      in, out, nb, cg, d, next, gates, static_cast<const T*>(src), static_cast<T*>(dst), dst_cap, n_out,
+      in, out, d, next, gates, static_cast<const T*>(src), static_cast<T*>(dst), dst_cap, n_out,
       dense.B, rule.use_eps, rule.eps, rule.wmax, L.smem_rows, static_cast<T*>(spill), dense, ctl, acc);
   return cudaGetLastError();
 }
@@ -403,22 +403,22 @@ RowsLaunch rows_launch(int P, int B, int esize, int sms) {
 }
 
 cudaError_t launch_rows_deal(int P, int grid, cudaStream_t s, const DevTable& src, uint64_t T,
-                             const PhaseBuckets& out, unsigned nb, unsigned cg, const PhaseDesc& d,
+                             const PhaseBuckets& out, const PhaseDesc& d,
                              const GateArgs* gates, const PhaseAcc& acc) {
   if (P == 1)
-    rows_deal_kernel<1><<<grid, kBlock, 0, s>>>(src.keys, src.alive, T, out, nb, cg, d, gates, acc);
+    rows_deal_kernel<1><<<grid, kBlock, 0, s>>>(src.keys, src.alive, T, out, d, gates, acc);
   else
-    rows_deal_kernel<2><<<grid, kBlock, 0, s>>>(src.keys, src.alive, T, out, nb, cg, d, gates, acc);
+    rows_deal_kernel<2><<<grid, kBlock, 0, s>>>(src.keys, src.alive, T, out, d, gates, acc);
   return cudaGetLastError();
 }
 
 cudaError_t launch_rows_phase(int P, const RowsLaunch& L, cudaStream_t s, const PhaseBuckets& in,
-                              const PhaseBuckets& out, unsigned nb, unsigned cg, const PhaseDesc& d,
+                              const PhaseBuckets& out, const PhaseDesc& d,
                               const PhaseDesc& next, const GateArgs* gates, const PhaseRule& rule,
                               const void* src, void* dst, uint64_t dst_cap, unsigned long long* n_out,
                               void* spill, const DevTable& dense, DevCtl* ctl, const PhaseAcc& acc) {
 #define PPR(PP, TT)                                                                                \
-  return launch_rows_pt<PP, TT>(L, s, in, out, nb, cg, d, next, gates, rule, src, dst, dst_cap, n_out, \
+  return launch_rows_pt<PP, TT>(L, s, in, out, d, next, gates, rule, src, dst, dst_cap, n_out, \
                                 spill, dense, ctl, acc)
   if (P == 1) {
     if (dense.f32) PPR(1, float);

@@ -97,16 +97,16 @@ int main(int argc, char** argv) {
     PhaseDesc d = {}, last_phase = {};
     d.count = 1;
     for (int P : {1, 2, 4, 6, 8})
-      say("phase", P, launch_phase(P, 12, nullptr, b, b, 1, 8, d, last_phase, nullptr, rule, t, nullptr, acc));
+      say("phase", P, launch_phase(P, 12, nullptr, b, b, d, last_phase, nullptr, rule, t, nullptr, acc));
     d.dense = 1;
     for (int P : {1, 2}) {
-      say("dense", P, launch_phase(P, 12, nullptr, b, b, 1, 8, d, last_phase, nullptr, rule, t, nullptr, acc));
+      say("dense", P, launch_phase(P, 12, nullptr, b, b, d, last_phase, nullptr, rule, t, nullptr, acc));
       for (int f32 = 0; f32 < 2; ++f32) {
         t.B = 256;
         t.f32 = f32;
         const RowsLaunch L = rows_launch(P, t.B, f32 ? 4 : 8, 152);
         say(f32 ? "rows32_" : "rows64_", P,
-            launch_rows_phase(P, L, nullptr, b, b, 1, 8, d, last_phase, nullptr, rule, nullptr, nullptr, 1,
+            launch_rows_phase(P, L, nullptr, b, b, d, last_phase, nullptr, rule, nullptr, nullptr, 1,
                               nullptr, nullptr, t, nullptr, acc));
       }
     }
