@@ -1336,6 +1336,7 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
       if (!ph.triangular) return PP_OK;
   Range range_("phases");
   const PhaseSizes z = phase_sizes(c, G, phases);
+  if (ppphase::nearly_full(T, z.est, c->n, phases)) return PP_OK;
   const size_t need = z.bytes;
   const double est = z.est;
   const int P32 = phase_words(c->n);

@@ -175,6 +175,24 @@ inline std::vector<Phase> plan(const std::vector<Gen>& gates, int W, const unsig
   return out;
 }
 
+// Whether a layer's table is so full that its classes are too: most of the 2^r
+// strings of a class are there, and the classes are few and uneven, a warp each.  On
+// the persistent kernel then, unless all phases are dense (a block's sweep takes full
+// classes best of all) or the table is small (a gate's barrier counts for more).
+// All-to-all Heisenberg layers, phases and persistent kernel, us: 10 qubits, 262144
+// strings (4^n / 4) 3120 and 1860; 12 qubits, 225 to 509 thousand (1.3 to 3 %) 5010
+// and 3700, 75 to 225 thousand 2400 and 2390; 14 qubits, 190 to 644 thousand (0.07 to
+// 0.2 %) 4220 and 4700; 8 qubits, 3280 to 16384 strings 680 and 890, 16384 to 16384
+// 605 and 520.
+constexpr uint64_t kFullTerms = 12288;
+constexpr double kFullShare = 1.0 / 32;
+inline bool nearly_full(uint64_t terms, double expected, int n, const std::vector<Phase>& phases) {
+  if (terms < kFullTerms || expected < kFullShare * std::pow(4.0, n)) return false;
+  for (const Phase& p : phases)
+    if (!p.triangular) return true;
+  return false;
+}
+
 // Buckets of one phase, and the records each has room for.
 struct Room {
   uint64_t nb = 0, cg = 0;

@@ -75,3 +75,28 @@ def test_batched_layers_are_phased(B, f32):
 def test_a_full_table_is_counted():
     r, _ = routes_of(pi.config1_ring(n=40, steps=5, eps=1e-5, max_weight=7), 0, room_factor=0.01)
     assert r["table_full"] > 0
+
+
+@pytest.mark.parametrize("n,eps,steps,last", [(9, 0.0, 3, False), (10, 0.0, 3, False), (10, 1e-6, 4, False),
+                                              (14, 2e-4, 3, True), (20, 1e-3, 3, True)])
+def test_full_tables_of_wide_classes_are_not_phased(n, eps, steps, last):
+    """All-to-all layers, whose phases are not dense, on tables that hold a large
+    share of the 4^n strings: the last layer is the persistent kernel's, at once and
+    not after a phase was given up; on more qubits it stays phased."""
+    wl = pi.config0_heisenberg(n, 0.05, steps)
+    wl.eps = eps
+    p = pp.Propagator.from_workload(wl, symmetry=0)
+    for layer in reversed(range(steps)):
+        before = pp.pp_debug_layer_routes(p.ctx)
+        gx, gz, th = wl.circuit.gate_arrays(layer)
+        p.apply_layer(gx, gz, th, True)
+    after = pp.pp_debug_layer_routes(p.ctx)
+    p.close()
+    assert after["phased"] - before["phased"] == int(last)
+    assert all(after[k] == before[k] for k in GIVEN_UP)
+
+
+@pytest.mark.parametrize("n", [8, 10])
+def test_full_tables_of_dense_phases_are(n):
+    r, entries = routes_of(pi.config1_ring(n=n, steps=8, eps=1e-6, max_weight=-1), 0)
+    assert entries > 4 ** n // 4 and r["phased"] == 8
