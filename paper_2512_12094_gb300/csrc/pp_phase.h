@@ -205,23 +205,42 @@ struct Workers {
   uint64_t least;
 };
 
-// For `strings` expected at the layer's end.  A bucket has room for four times its
-// share and more, since classes come in lumps.
-inline Room bucket_room(double strings, const Workers& w, double factor) {
+// Strings expected at the end of a layer, and what a bucket may meet of them.
+struct Expected {
+  double strings;  // that buckets are made for
+  double lumps;    // the growth of the layer before, extrapolated
+};
+
+// The next growth is a quarter above the last one, as far as that goes: one term
+// becomes thousands in the first layer of an all-to-all circuit, and the tables
+// after it ten times as many each, not thousands of times.  (Buckets for all of the
+// extrapolation: 4 GB for the 16384 strings of 8 qubits, 20 GB for 75 thousand of 12,
+// whose counters a warp goes through one after the other.)  Nor are there more strings
+// than `possible`.
+constexpr double kMostGrowth = 32.0;
+inline Expected expected(uint64_t terms, double last_growth, double possible) {
+  const double grown = (double)terms * (1.25 * last_growth > 1.5 ? 1.25 * last_growth : 1.5);
+  const double most = std::fmin((double)terms * kMostGrowth, possible);
+  return {std::fmin(grown, most), grown};
+}
+
+// A bucket has room for four times its share and more, since classes come in lumps:
+// up to four times `fill` where the table is growing fast.
+inline Room bucket_room(const Expected& e, const Workers& w, double factor) {
   Room r;
-  const uint64_t n = (uint64_t)std::ceil(strings * factor / w.fill);
-  r.nb = n > w.least ? n : w.least;
-  r.cg = (256 + (uint64_t)(4.0 * strings / (double)r.nb)) / 8 * 8;
+  r.nb = (uint64_t)std::ceil(std::fmin(e.strings * factor / w.fill, 1e12));
+  if (r.nb < w.least) r.nb = w.least;
+  r.cg = (256 + (uint64_t)(4.0 * std::fmin(e.lumps / (double)w.least, w.fill / factor))) / 8 * 8;
   return r;
 }
 
 // Each phase's, by what takes its buckets.  (With the buckets of the blocks for all,
 // all-to-all layers with truncation, whose phases are not dense, ran on 304 of 1824
 // warps; with those of the warps for all, a dense phase takes many times the parts.)
-inline std::vector<Room> bucket_rooms(const std::vector<Phase>& phases, double strings, const Workers& dense,
+inline std::vector<Room> bucket_rooms(const std::vector<Phase>& phases, const Expected& e, const Workers& dense,
                                       const Workers& sparse, double factor) {
   std::vector<Room> out;
-  for (const Phase& p : phases) out.push_back(bucket_room(strings, p.triangular ? dense : sparse, factor));
+  for (const Phase& p : phases) out.push_back(bucket_room(e, p.triangular ? dense : sparse, factor));
   return out;
 }
 
