@@ -137,4 +137,18 @@ inline int share_units(int slots, int64_t running, double wanted, int units_free
   return std::min(want, units_free);
 }
 
+// May a running job hold `extra` bytes on top of the reservations for the time of a
+// layer, that its layer is faster with but can do without?  Only memory that nobody
+// else could have in that time: none while a running job waits to grow, and none
+// that a queued job which fits now, and for which a slot is free, would be kept out
+// by.
+inline bool may_lend(size_t budget, size_t reserved, size_t extra, int64_t growing, int64_t running, int slots,
+                     const std::vector<size_t>& queued) {
+  if (growing > 0 || extra > budget || reserved > budget - extra) return false;
+  if (running >= slots) return true;
+  for (const size_t r : queued)
+    if (r <= budget - reserved && r > budget - reserved - extra) return false;
+  return true;
+}
+
 }  // namespace ppadm

@@ -18,6 +18,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <mutex>
 #include <string>
@@ -186,6 +187,8 @@ struct pp_ctx {
   int phase_fails = 0;         // phased layers given up in a row
   int phase_gates = kPhaseGates;  // of a phase at most
   int64_t routes[PP_ROUTES] = {};
+  std::function<bool(size_t)> take_scratch;  // set_scratch_hooks
+  std::function<void()> give_scratch;
   float* h_activity = nullptr; // pinned, kActivityMax gates
   void* sort_scratch = nullptr;  // scratch of the sort-based merge (merge_method 1)
   size_t sort_scratch_bytes = 0;
@@ -1353,16 +1356,22 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   auto al = align256;
   const size_t clear = z.clear;
   if (z.most >= (1ull << 26) || need > kPhaseBytesMax) return PP_OK;
-  if (c->cfg.mem_budget_bytes && c->bytes + need > c->cfg.mem_budget_bytes) return PP_OK;
-  unsigned char* scratch = nullptr;
-  if (dmalloc(c, (void**)&scratch, need) != PP_OK) {  // no room for it: the other path
-    cudaGetLastError();
-    return PP_OK;
+  bool lent = false;  // the scratch is beyond the budget, by the owner's leave
+  if (c->cfg.mem_budget_bytes && c->bytes + need > c->cfg.mem_budget_bytes) {
+    if (!c->take_scratch || !c->take_scratch(c->bytes + need)) return PP_OK;
+    lent = true;
   }
+  unsigned char* scratch = nullptr;
   auto release = [&](pp_status st) {
     dfree(c, scratch, need);
+    if (lent) c->give_scratch();
     return st;
   };
+  if (dmalloc(c, (void**)&scratch, need) != PP_OK) {  // no room for it: the other path
+    cudaGetLastError();
+    scratch = nullptr;
+    return release(PP_OK);
+  }
   PhaseAcc acc;
   acc.st = reinterpret_cast<PhaseStat*>(scratch);
   acc.delta = reinterpret_cast<long long*>(acc.st + 1);
@@ -2457,12 +2466,7 @@ double ppk::layer_fraction_wanted(const pp_ctx* c) {
   return std::min(1.0, (double)layer_grid_want(c, c->n_terms) / full);
 }
 
-size_t ppk::layer_scratch_bytes(const pp_ctx* c, int n_gates) {
-  if (!c || c->batched || !c->cfg.layer_kernel || c->layer_bps <= 0 || !phases_allowed(c) ||
-      n_gates < kPhaseMinGates)
-    return 0;
-  ppphase::Phase kind;
-  kind.triangular = dense_classes(c);
-  const size_t bytes = phase_sizes(c, (size_t)n_gates, std::vector<ppphase::Phase>(kPhaseMax, kind)).bytes;
-  return bytes > kPhaseBytesMax ? 0 : bytes;
+void ppk::set_scratch_hooks(pp_ctx* c, std::function<bool(size_t)> take, std::function<void()> give) {
+  c->take_scratch = std::move(take);
+  c->give_scratch = std::move(give);
 }

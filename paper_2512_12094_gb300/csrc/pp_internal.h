@@ -6,6 +6,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <functional>
 #include <string>
 
 namespace ppk {
@@ -354,9 +355,11 @@ void set_grid_fraction(pp_ctx* c, double frac);
 // The fraction of the GPU's co-resident blocks the context's next persistent
 // layer launch would use with no limit (0 when it has no persistent path).
 double layer_fraction_wanted(const pp_ctx* c);
-// Device memory beyond what it holds that the context's next layer of n_gates
-// gates could use while it runs (0: none; it does without where there is none).
-size_t layer_scratch_bytes(const pp_ctx* c, int n_gates);
+// For a context with a memory budget whose owner has more.  A layer whose plan is
+// phased and whose scratch passes the budget asks take(bytes the context would hold in
+// all); if that is granted the scratch is used beyond the budget, which stays as it
+// is for everything else, and give() follows once the scratch is freed.
+void set_scratch_hooks(pp_ctx* c, std::function<bool(size_t)> take, std::function<void()> give);
 
 // ------------------------------------------------------- batched launchers
 // Same contracts as the single-column kernels above, on B-column rows.

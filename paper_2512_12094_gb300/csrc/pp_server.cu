@@ -20,7 +20,9 @@
 // reservation and asks the server for more before the next layer; a layer
 // that still runs out of room (PP_ERR_CAPACITY, the context restored to its
 // state before the layer) gets twice the reservation and is applied again.
-// The job never starts over.  A running job waiting for more memory has
+// The job never starts over.  The scratch of a layer applied as phases, with which it
+// runs several times faster, is lent on top of the reservation for as long as it is
+// in use, if nobody else needs the memory.  A running job waiting for more memory has
 // priority over queued jobs; a queued job that younger jobs have passed
 // kMaxBypass times is passed no more.  If every running job waits for memory
 // the one that notices gives its memory back and is queued again at the head
@@ -61,6 +63,7 @@ struct Job {
   int n_layers = 0;
   int boundary = 1;
   size_t reserve = 0;
+  size_t lent = 0;   // held on top of it while a phased layer has its scratch
   int grows = 0;     // reservation increases
   int restarts = 0;  // times the job gave its memory back and started over
   int bypassed = 0;  // younger jobs admitted while this one waited at the queue's head
@@ -209,15 +212,29 @@ Grow grow_reservation(pp_server* s, Job& j, size_t want) {
   }
 }
 
-// Raise a running job's reservation to `want` if the memory is free at once (for
-// what a layer can do without).
-bool try_grow_reservation(pp_server* s, Job& j, size_t want) {
+// Lend a running job what its context would hold beyond its reservation with the
+// scratch of a phased layer in hand, if nobody else needs it (ppadm::may_lend).  The
+// reservation itself, the context's budget and what a later increase starts from stay
+// as they are.
+bool lend(pp_server* s, Job& j, size_t total) {
   std::lock_guard<std::mutex> lock(s->mu);
-  if (want <= j.reserve || s->growing > 0 || s->reserved - j.reserve + want > s->budget) return false;
-  s->reserved += want - j.reserve;
-  j.reserve = want;
-  j.grows++;
+  const size_t want = round_mib((double)total);
+  if (want <= j.reserve) return true;
+  std::vector<size_t> queued;
+  for (const auto& q : s->queue) queued.push_back(q->reserve);
+  const size_t extra = want - j.reserve;
+  if (!ppadm::may_lend(s->budget, s->reserved, extra, s->growing, s->running, s->slots, queued)) return false;
+  s->reserved += extra;
+  j.lent = extra;
   return true;
+}
+
+void give_back_lent(pp_server* s, Job& j) {
+  std::lock_guard<std::mutex> lock(s->mu);
+  if (!j.lent) return;
+  s->reserved -= j.lent;
+  j.lent = 0;
+  s->cv_work.notify_all();
 }
 
 // Run one job on `stream`: returns its status; fills r.  *give_back is set
@@ -254,6 +271,10 @@ pp_status run_job(pp_server* s, Job& j, cudaStream_t stream, pp_job_result& r, b
                    j.coef.data(), &ctx);
     if (st != PP_ERR_CAPACITY || !grow_or_stop(st)) break;
   }
+  if (ctx) {
+    ppk::set_scratch_hooks(ctx, [s, &j](size_t total) { return lend(s, j, total); },
+                           [s, &j] { give_back_lent(s, j); });
+  }
   int64_t live_prev = -1;
   for (int l = 0; st == PP_OK && l < j.n_layers; ++l) {
     // proactive: the memory the context holds, scaled by the live-term
@@ -273,11 +294,6 @@ pp_status run_job(pp_server* s, Job& j, cudaStream_t stream, pp_job_result& r, b
           break;
         }
       }
-      // scratch with which the layer runs as phases, several times faster; the
-      // copy of the table that a budgeted layer keeps comes on top of it
-      const size_t scratch = ppk::layer_scratch_bytes(ctx, (int)j.gates.size());
-      if (scratch && try_grow_reservation(s, j, round_mib((double)(2 * stats.device_bytes + scratch))))
-        pp_set_budget(ctx, j.reserve);
     }
     for (;;) {
       // A layer runs in one persistent launch on the share units it holds

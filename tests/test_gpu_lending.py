@@ -1,0 +1,86 @@
+"""A server lends the scratch of phased layers beside the reservations: it comes back
+after the layer, keeps nobody waiting and restarts nobody (needs a GB300)."""
+import time
+
+import numpy as np
+import pytest
+
+import paper_2512_12094_gb300 as pp
+import pp_inputs as pi
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    pp.build()
+    pp.load()
+
+
+def ring_job(n=32, steps=8, eps=1e-4, mem_bytes=0, **cfg):
+    wl = pi.config1_ring(n=n, steps=steps, eps=eps, max_weight=8, symmetry=1)
+    c = pp.pp_config_default(n_qubits=n, symmetry=1, coeff_eps=eps, max_weight=8, **cfg)
+    x, z, co = wl.observable.arrays()
+    gx, gz, th = wl.circuit.gate_arrays(0)
+    return pp.make_job(c, x, z, co, pp.pack_gates(gx, gz), th, steps, wl.state.bloch, True, mem_bytes)
+
+
+def serve(jobs, slots, budget):
+    """(results, largest sum of reservations seen)"""
+    server = pp.pp_server_create(slots, budget, 0)
+    ids = [pp.pp_submit(server, j) for j, _ in jobs]
+    most = 0
+    while True:
+        st = pp.pp_server_stats(server)
+        most = max(most, st["reserved_bytes"])
+        if st["completed"] == len(jobs):
+            break
+        time.sleep(2e-4)
+    res = [pp.pp_server_wait(server, i) for i in ids]
+    assert pp.pp_server_stats(server)["reserved_bytes"] == 0
+    pp.pp_server_destroy(server)
+    assert all(r["status"] == 0 for r in res), [r["message"] for r in res]
+    return res, most
+
+
+def test_reservations_without_the_scratch():
+    """What a job holds when it ends is what it holds with the persistent kernel, up
+    to the table's growth, which each way extrapolates from its own layers; the
+    buckets of its phases (5 MB at least) are not in it.  While a layer runs they
+    are."""
+    (a,), most = serve([ring_job(steps=5)], 2, 4 << 30)
+    (b,), _ = serve([ring_job(steps=5, block_threads=256)], 2, 4 << 30)
+    assert a["value"] == pytest.approx(b["value"], abs=1e-10)
+    assert a["reserved_bytes"] <= b["reserved_bytes"] + (4 << 20) and a["restarts"] == 0
+    assert most >= a["reserved_bytes"]
+
+
+@pytest.mark.parametrize("budget_mib", [40, 80, 160, 400])
+def test_tight_budgets_restart_nobody_more(budget_mib):
+    """Eight jobs in four slots, whose tables and scratch do not all fit: no more jobs
+    start over than with the persistent kernel, and reservations stay in the budget."""
+    budget = budget_mib << 20
+    kinds = [dict(n=32, steps=9), dict(n=24, steps=8), dict(n=40, steps=7), dict(n=16, steps=6)] * 2
+    a, most = serve([ring_job(**k) for k in kinds], 4, budget)
+    b, _ = serve([ring_job(block_threads=256, **k) for k in kinds], 4, budget)
+    assert most <= budget
+    for u, v in zip(a, b):
+        assert u["value"] == pytest.approx(v["value"], abs=1e-10)
+    assert sum(r["restarts"] for r in a) <= sum(r["restarts"] for r in b) + 1
+
+
+def test_a_queued_job_does_not_wait_for_scratch():
+    """A long job runs; a short one whose reservation fits beside the long one's, but
+    not beside its buckets (5 MB at least), starts before the long one is done."""
+    long_job, kl = ring_job(n=32, steps=2000, eps=1e-2, mem_bytes=4 << 20)
+    short, ks = ring_job(n=16, steps=3, eps=1e-3, mem_bytes=35 << 20)
+    server = pp.pp_server_create(2, 40 << 20, 0)
+    i = pp.pp_submit(server, long_job)
+    time.sleep(0.02)
+    k = pp.pp_submit(server, short)
+    rs = pp.pp_server_wait(server, k)
+    rl = pp.pp_server_wait(server, i)
+    pp.pp_server_destroy(server)
+    assert rs["status"] == 0 and rl["status"] == 0
+    assert rl["run_ms"] > 40.0 and rl["reserved_bytes"] == 4 << 20
+    assert rs["latency_ms"] < rl["run_ms"] / 2
