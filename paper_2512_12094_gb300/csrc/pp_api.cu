@@ -504,10 +504,6 @@ pp_status ensure_capacity(pp_ctx* c, uint64_t need) {
   return PP_OK;
 }
 
-// Strings of n qubits, where that may be less than what a table holds.
-constexpr int kCountedQubits = 20;
-uint64_t strings_there_are(const pp_ctx* c) { return c->n <= kCountedQubits ? 1ull << (2 * c->n) : ~0ull; }
-
 // Make room before (or in the middle of) a layer: drop truncated entries when
 // they are a quarter of the table or more, then make sure the capacity holds
 // factor x the entries.  The caller derives factor from how much the previous
@@ -522,7 +518,7 @@ pp_status make_room(pp_ctx* c, uint64_t factor = 2) {
   // no table needs more than twice the strings there are: a growth extrapolated
   // from a first layer of a few terms is gigabytes otherwise, whose index every
   // compaction clears (three layers on 8 qubits: 3 GB and 3.2 ms; so 10 MB and 3.0)
-  const uint64_t most = c->n <= kCountedQubits ? 2 * strings_there_are(c) : ~0ull;
+  const uint64_t most = c->n <= 20 ? 2ull << (2 * c->n) : ~0ull;
   if (std::min(factor * c->n_terms, most) <= cap) return PP_OK;
   const uint64_t least = std::min(c->n_terms * 4, most);
   const uint64_t generous = std::max<uint64_t>(least, std::min(factor * c->n_terms * 3 / 2, most));
@@ -1283,8 +1279,7 @@ PhaseSizes phase_sizes(const pp_ctx* c, size_t G, const std::vector<ppphase::Pha
   PhaseSizes z;
   const int P32 = phase_words(c->n);
   const size_t P = phases.size();
-  const ppphase::Expected e = ppphase::expected(
-      c->n_terms, c->last_growth, (double)std::min(strings_there_are(c), c->buf[c->active].cap));
+  const ppphase::Expected e = ppphase::expected(c->n_terms, c->last_growth, (double)c->buf[c->active].cap);
   z.est = e.strings;
   const ppphase::Workers warps = {0.5 * phase_strings_per_warp(P32), (uint64_t)c->sms * phase_warps_per_sm()};
   const ppphase::Workers blocks = c->batched ? ppphase::Workers{kRowsFill, (uint64_t)c->sms * 8}

@@ -181,11 +181,12 @@ inline std::vector<Phase> plan(const std::vector<Gen>& gates, int W, const unsig
 // classes best of all) or the table is small (a gate's barrier counts for more).
 // All-to-all Heisenberg layers, phases and persistent kernel, us: 10 qubits, 262144
 // strings (4^n / 4) 3120 and 1860; 12 qubits, 225 to 509 thousand (1.3 to 3 %) 5010
-// and 3700, 75 to 225 thousand 2400 and 2390; 14 qubits, 190 to 644 thousand (0.07 to
-// 0.2 %) 4220 and 4700; 8 qubits, 3280 to 16384 strings 680 and 890, 16384 to 16384
-// 605 and 520.
-constexpr uint64_t kFullTerms = 12288;
-constexpr double kFullShare = 1.0 / 32;
+// and 3700, 75 to 225 thousand 2400 and 2390; 14 qubits, 190 to 644 thousand (1 %
+// expected) 4220 and 4700; a 3 x 4 torus, 23 to 101 thousand (2.4 % expected), given up
+// after 2500, 690; 8 qubits, 3280 to 16384 strings 680 and 890, 16384 to 16384
+// 605 and 520; a ring of 9 qubits, 8505 to 118821 446 and 385.
+constexpr uint64_t kFullTerms = 8192;
+constexpr double kFullShare = 1.0 / 64;
 inline bool nearly_full(uint64_t terms, double expected, int n, const std::vector<Phase>& phases) {
   if (terms < kFullTerms || expected < kFullShare * std::pow(4.0, n)) return false;
   for (const Phase& p : phases)
@@ -216,7 +217,7 @@ struct Expected {
 // after it ten times as many each, not thousands of times.  (Buckets for all of the
 // extrapolation: 4 GB for the 16384 strings of 8 qubits, 20 GB for 75 thousand of 12,
 // whose counters a warp goes through one after the other.)  Nor are there more strings
-// than `possible`.
+// than the tables hold, which is `possible`.
 constexpr double kMostGrowth = 32.0;
 inline Expected expected(uint64_t terms, double last_growth, double possible) {
   const double grown = (double)terms * (1.25 * last_growth > 1.5 ? 1.25 * last_growth : 1.5);

@@ -48,8 +48,8 @@ def test_fill_and_room(rooms, terms, factor, kind, fill, least):
     (100, 1e9, 1e18, 3200), (10 ** 9, 1e9, 1e18, 32e9), (100, 2.0, 120, 120)])
 def test_a_growth_is_extrapolated_so_far(rooms, terms, growth, possible, want):
     """A first layer that multiplies one term by thousands says nothing of the kind
-    about the next, and no layer ends with more strings than there are: 4^n on few
-    qubits, or what the tables hold."""
+    about the next, and no layer ends with more strings than the tables hold (whose
+    room stops at twice the 4^n strings there are)."""
     strings, sizes = rooms(terms, [0, 1], growth, possible)
     assert strings == pytest.approx(want, rel=1e-12)
     for (nb, cg), fill, least in zip(sizes, (368, 700), (1824, 304)):
