@@ -185,7 +185,8 @@ struct pp_ctx {
   double phase_room = 1.0;     // buckets per layer relative to the default sizing
   int phase_wait = 0;          // layers left before phases are tried again
   int phase_fails = 0;         // phased layers given up in a row
-  int phase_gates = kPhaseGates;  // of a phase at most
+  bool rank_bound = false;     // dense phases are cut so that no class can outgrow its room,
+  bool class_bound = false;    // and the others
   int64_t routes[PP_ROUTES] = {};
   std::function<bool(size_t)> take_scratch;  // set_scratch_hooks
   std::function<void()> give_scratch;
@@ -1327,10 +1328,14 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   if (ent.activity.size() != G) ent.activity.assign(G, kPhaseGuess);
   const bool dense = dense_classes(c);
   ppphase::Limits lim;
-  lim.max_gates = c->phase_gates;
   lim.max_active = c->phase_active;
   lim.max_bits = kPhaseBits;
   lim.triangular = dense;
+  if (c->rank_bound) lim.max_gates = kPhaseRank;
+  if (c->class_bound) {
+    lim.max_plain = 63 - __builtin_clzll((uint64_t)phase_strings_per_warp(phase_words(c->n)));
+    lim.max_bits = std::min(kPhaseBits, lim.max_plain);
+  }
   const std::vector<ppphase::Phase> phases =
       ppphase::plan(gens, c->W, touch.data(), ent.activity.data(), lim);
   const size_t P = phases.size();
@@ -1501,17 +1506,18 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   if (const unsigned why = c->h_ctl->stall) {
     // given up: the input table is whole (its index may not be).  Next time
     // with finer phases or more buckets, and after ever longer waits.
-    c->routes[(why & kPhaseClassFull)    ? PP_ROUTE_CLASS_FULL
+    const unsigned classes = kPhaseClassFull | kPhaseRankFull;
+    c->routes[(why & classes)            ? PP_ROUTE_CLASS_FULL
               : (why & kPhaseBucketFull) ? PP_ROUTE_BUCKET_FULL
                                          : PP_ROUTE_TABLE_FULL]++;
-    if (why & kPhaseClassFull) {
-      // a dense class of more active gates than its room (a star of bonds):
-      // then no phase has more gates than that
-      if (dense && c->phase_gates > kPhaseRank)
-        c->phase_gates = kPhaseRank;
-      else
-        c->phase_active = std::max(0.5, 0.6 * c->phase_active);
-    }
+    // a class of more active gates than its room (a star of bonds), or of more
+    // strings: then phases have no more gates, or touch no more bits, than a class has
+    // room for, and it does not happen again (dense ones in either case: where a warp's
+    // class is too large a block's is soon)
+    if ((why & classes) && c->rank_bound && (c->class_bound || !(why & kPhaseClassFull)))
+      c->phase_active = std::max(0.5, 0.6 * c->phase_active);
+    if (why & classes) c->rank_bound = true;
+    if (why & kPhaseClassFull) c->class_bound = true;
     if (why & kPhaseBucketFull) {
       c->phase_room = std::min(8.0, 2.0 * c->phase_room);
       c->phase_active = std::max(0.5, 0.8 * c->phase_active);

@@ -254,6 +254,7 @@ enum : unsigned {
   kPhaseBucketFull = 1u,
   kPhaseClassFull = 2u,  // one class outgrew a warp's shared memory
   kPhaseTableFull = 4u,  // the destination table
+  kPhaseRankFull = 16u,  // a dense class has more than kPhaseRank active gates
 };
 
 struct alignas(16) PhaseStat {

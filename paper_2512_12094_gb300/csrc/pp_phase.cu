@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(kPT, kPBlocks)
     for (int k = lane; k < kSlots / 2; k += 32) reinterpret_cast<unsigned*>(S.slot)[k] = 0u;
     for (int k = lane; k < kPhaseGates; k += 32) S.acdl[k] = 0;
     __syncwarp();
-    unsigned uni = 0;
+    unsigned uni = 0, all = ~0u, any = 0;
     int n = 0;
     constexpr int U = PhaseDims<P>::kLoads;
     for (int i0 = 0; i0 < cnt; i0 += 32 * U) {
@@ -408,6 +408,8 @@ __global__ void __launch_bounds__(kPT, kPBlocks)
         n += __popc(bal);
         if (mine) {
           uni |= m[u].x;
+          all &= m[u].y;
+          any |= m[u].y;
           if (p < C) {
             S.key[p] = K[u];
             S.coef[p] = c[u];
@@ -419,6 +421,8 @@ __global__ void __launch_bounds__(kPT, kPBlocks)
     uni = __reduce_or_sync(kFull, uni);
     __syncwarp();
     const bool too_many = n > C;
+    // one class, which no further bit of its hash divides
+    if (too_many && __reduce_and_sync(kFull, all) == __reduce_or_sync(kFull, any)) s = kMaxSplit;
     n = phase_gates<P>(S, B.gate, d, rule, too_many ? 0 : n, uni);
     if (too_many) n = -1;
     const bool ok = n >= 0;
@@ -732,7 +736,7 @@ __global__ void __launch_bounds__(kDT, 2)
       const bool fits = laid && S.slots <= kDSlots && S.orders <= kDOrder;
       if (!fits) {  // uniform
         if (S.bad || ++s > kMaxSplit) {
-          fail |= kPhaseClassFull;
+          fail |= S.bad ? kPhaseRankFull : kPhaseClassFull;
           break;
         }
         continue;

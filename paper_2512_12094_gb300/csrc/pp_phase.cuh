@@ -7,7 +7,9 @@
 namespace ppk {
 namespace {
 
-constexpr int kMaxSplit = 10;   // a bucket is cut into at most 2^kMaxSplit parts
+// A bucket is cut into at most 2^kMaxSplit parts.  Two classes that only just fit a
+// part each must not meet in one: with 10 bits they did in some bucket of thousands.
+constexpr int kMaxSplit = 16;
 
 template <int P>
 struct alignas(P == 1 ? 8 : 16) PKey {

@@ -66,6 +66,7 @@ inline std::vector<unsigned char> touched(const std::vector<Gen>& gates, int W, 
 // How a layer is cut.
 struct Limits {
   int max_gates = kMaxGates;  // per phase
+  int max_plain = kMaxGates;  // of commuting ones that are not triangular
   double max_active = 3.0;    // mean number of its gates active on a string
   int max_bits = 10;          // key bits a phase that does not commute may touch
   bool triangular = false;    // dense classes are possible: look for triangular runs
@@ -87,7 +88,8 @@ inline std::vector<Phase> plan(const std::vector<Gen>& gates, int W, const unsig
                                const float* activity, const Limits& lim) {
   std::vector<Phase> out;
   const int G = (int)gates.size();
-  const int max_gates = lim.max_gates < kMaxGates ? lim.max_gates : kMaxGates;
+  const int most[2] = {lim.max_plain < kMaxGates ? lim.max_plain : kMaxGates,
+                       lim.max_gates < kMaxGates ? lim.max_gates : kMaxGates};
   int run_end = 0;        // of the commuting run that g is in
   double part_act = 0.0;  // activity of one of its parts
   for (int g = 0; g < G;) {
@@ -117,7 +119,7 @@ inline std::vector<Phase> plan(const std::vector<Gen>& gates, int W, const unsig
     double act = 0.0;
     for (; c < run_end && c - g < kMaxGates; ++c) {
       if (!touch[c]) continue;
-      if (nc >= max_gates || (nc > 0 && act + 0.5 * activity[c] > part_act)) break;
+      if (nc >= most[tri] || (nc > 0 && act + 0.5 * activity[c] > part_act)) break;
       if (tri) {
         bool keeps = true;
         for (size_t k = 0; k < own.size() && keeps; k += 2 * W) {
@@ -184,8 +186,9 @@ inline std::vector<Phase> plan(const std::vector<Gen>& gates, int W, const unsig
 // and 3700, 75 to 225 thousand 2400 and 2390; 14 qubits, 190 to 644 thousand (1 %
 // expected) 4220 and 4700; a 3 x 4 torus, 23 to 101 thousand (2.4 % expected), given up
 // after 2500, 690; 8 qubits, 3280 to 16384 strings 680 and 890, 16384 to 16384
-// 605 and 520; a ring of 9 qubits, 8505 to 118821 446 and 385.
-constexpr uint64_t kFullTerms = 8192;
+// 605 and 520; tori of 3 x 3, 12 to 25 thousand 910 and 530, 8590 to 9410 strings 220
+// and 490.
+constexpr uint64_t kFullTerms = 11000;
 constexpr double kFullShare = 1.0 / 64;
 inline bool nearly_full(uint64_t terms, double expected, int n, const std::vector<Phase>& phases) {
   if (terms < kFullTerms || expected < kFullShare * std::pow(4.0, n)) return false;

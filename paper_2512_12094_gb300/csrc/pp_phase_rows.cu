@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(256)
       const bool fits = n <= kRStrings && !S.bad;
       if (!fits) {  // uniform
         if (S.bad || ++s > kMaxSplit) {
-          fail |= kPhaseClassFull;
+          fail |= S.bad ? kPhaseRankFull : kPhaseClassFull;
           break;
         }
         continue;

@@ -100,3 +100,25 @@ def test_full_tables_of_wide_classes_are_not_phased(n, eps, steps, last):
 def test_full_tables_of_dense_phases_are(n):
     r, entries = routes_of(pi.config1_ring(n=n, steps=8, eps=1e-6, max_weight=-1), 0)
     assert entries > 4 ** n // 4 and r["phased"] == 8
+
+
+@pytest.mark.parametrize("lx,ly,steps", [(5, 5, 7), (6, 6, 6)])
+def test_classes_outgrow_their_room_once_of_a_kind(lx, ly, steps):
+    """Bonds of every site without a weight limit: a layer of a large table is given
+    up for a class of more than ten active gates, or of more strings than a warp holds;
+    the layers after it are cut so that no class can be, and are phased again."""
+    wl = pi.torus_ising(lx, ly, steps, 0.4, 0.6, 0.3, 2e-4, -1, pp.sym_torus(lx))
+    p = pp.Propagator.from_workload(wl, symmetry=wl.symmetry)
+    b = pp.Propagator.from_workload(wl, symmetry=wl.symmetry, block_threads=256)
+    seen = []
+    for layer in reversed(range(steps)):
+        gx, gz, th = wl.circuit.gate_arrays(layer)
+        p.apply_layer(gx, gz, th, True)
+        b.apply_layer(gx, gz, th, True)
+        assert p.num_terms()[0] == b.num_terms()[0]
+        seen.append(pp.pp_debug_layer_routes(p.ctx))
+    p.close()
+    b.close()
+    assert 1 <= seen[-1]["class_full"] <= 2
+    assert seen[-1]["phased"] == seen[-2]["phased"] + 1 or seen[-1]["class_full"] == seen[-2]["class_full"] + 1
+    assert sum(r["class_full"] == 1 for r in seen) > 1  # it is not every layer's lot
