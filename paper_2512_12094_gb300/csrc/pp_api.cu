@@ -1336,10 +1336,10 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
     lim.max_plain = 63 - __builtin_clzll((uint64_t)phase_strings_per_warp(phase_words(c->n)));
     lim.max_bits = std::min(kPhaseBits, lim.max_plain);
   }
-  const std::vector<ppphase::Phase> phases =
-      ppphase::plan(gens, c->W, touch.data(), ent.activity.data(), lim);
+  lim.max_phases = std::min<size_t>(kPhaseMax, n_touch / kPhaseMinGates);
+  const std::vector<ppphase::Phase> phases = ppphase::plan(gens, c->W, touch.data(), ent.activity.data(), lim);
   const size_t P = phases.size();
-  if (P == 0 || P > (size_t)kPhaseMax || P * kPhaseMinGates > n_touch) return PP_OK;
+  if (P == 0 || P > lim.max_phases) return PP_OK;
   if (c->batched)
     for (const ppphase::Phase& ph : phases)
       if (!ph.triangular) return PP_OK;

@@ -70,6 +70,7 @@ struct Limits {
   double max_active = 3.0;    // mean number of its gates active on a string
   int max_bits = 10;          // key bits a phase that does not commute may touch
   bool triangular = false;    // dense classes are possible: look for triangular runs
+  size_t max_phases = ~(size_t)0;  // the plan stops at one more
 };
 
 // Cut the gates into phases, greedily.  Gates that touch nothing are in no
@@ -77,8 +78,8 @@ struct Limits {
 //
 // A run of commuting gates (up to the first that does not commute with all
 // before it) is cut into equal parts in which at most max_active gates are active
-// on a string on average (activity: the mean per gate, from the layer before):
-// classes grow with the number of active gates, and a class has to fit one block.
+// on a string on average (activity: per gate, from the layer before): classes grow
+// with the number of active gates, and a class has to fit one block.
 // With `triangular` a part also ends where a gate would leave an earlier one
 // without a bit of its own.  Parts of fewer than kShortRun gates give way to a run
 // whose generators touch at most max_bits key bits (at most 2^max_bits strings
@@ -92,7 +93,7 @@ inline std::vector<Phase> plan(const std::vector<Gen>& gates, int W, const unsig
                        lim.max_gates < kMaxGates ? lim.max_gates : kMaxGates};
   int run_end = 0;        // of the commuting run that g is in
   double part_act = 0.0;  // activity of one of its parts
-  for (int g = 0; g < G;) {
+  for (int g = 0; g < G && out.size() <= lim.max_phases;) {
     if (!touch[g]) {
       ++g;
       continue;

@@ -31,3 +31,14 @@ def test_no_phase_passes_the_bound(driver, n, gates, support, tri, plain, bits):
         assert len(kinds) == 3 and all(k.isdigit() for k in kinds), got
         total = [a + int(b) for a, b in zip(total, kinds)]
     assert sum(total) > 5 and (tri or total[2] == 0)
+
+
+@pytest.mark.parametrize("n", [3, 8, 20, 64])
+@pytest.mark.parametrize("limit", [0, 1, 64, 10000])
+def test_a_plan_of_too_many_phases_stops(tmp_path_factory, n, limit):
+    exe = str(tmp_path_factory.mktemp("stop") / "stop")
+    subprocess.run(["g++", "-O1", "-std=c++17", "-Wall", "-Werror", "-fsanitize=address,undefined",
+                    os.path.join(HERE, "phase_stop_main.cpp"), "-o", exe], check=True)
+    out = subprocess.run([exe, str(n), str(limit)], capture_output=True, text=True, check=True).stdout
+    whole, part, same = map(int, out.split())
+    assert part == min(whole, limit + 1) and same
