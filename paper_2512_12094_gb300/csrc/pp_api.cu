@@ -96,9 +96,7 @@ struct ArgsEntry {
   GateArgs* d_args = nullptr;      // device copy
   size_t n = 0;                    // its size in bytes
   uint64_t last_use = 0;
-  // mean number of live strings of a gate's table that anticommuted with it in
-  // the last layer, per gate (apply_layer_phased)
-  std::vector<float> activity;
+  std::vector<float> activity;  // PhaseAcc::activity of the last layer (apply_layer_phased)
 };
 
 struct GraphEntry {
@@ -1337,7 +1335,17 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
     lim.max_bits = std::min(kPhaseBits, lim.max_plain);
   }
   lim.max_phases = std::min<size_t>(kPhaseMax, n_touch / kPhaseMinGates);
-  const std::vector<ppphase::Phase> phases = ppphase::plan(gens, c->W, touch.data(), ent.activity.data(), lim);
+  std::vector<ppphase::Phase> phases = ppphase::plan(gens, c->W, touch.data(), ent.activity.data(), lim);
+  if (phases.size() > lim.max_phases) {
+    // a layer that grew many times over leaves activities above one, and no phase of
+    // two gates after it: they are shares at most
+    bool above = false;
+    for (float& a : ent.activity) {
+      above |= a > 1.0f;
+      a = std::min(a, 1.0f);
+    }
+    if (above) phases = ppphase::plan(gens, c->W, touch.data(), ent.activity.data(), lim);
+  }
   const size_t P = phases.size();
   if (P == 0 || P > lim.max_phases) return PP_OK;
   if (c->batched)

@@ -273,7 +273,14 @@ struct PhaseAcc {
   unsigned long long* ac;  // [gates] live anticommuting strings
   unsigned* touch;         // [gates] some string may anticommute (or be damped)
   unsigned* seen;          // [gates] of dense phases: strings of the counted buckets active in it
-  float* activity;         // [gates] ac / live, written by launch_phase_end
+  // [gates] strings active in it, of a dense phase those that enter the phase, per live
+  // string: of those that enter the gate, not counting what dense phases before it
+  // added.  So the later gates of a growing layer count for more than their share and
+  // are cut into shorter phases, whose classes are fewer and larger than the layer's
+  // first.  With the share of the strings that enter the phase instead, and limits of
+  // 1.5 to 8 (kPhaseActive), no limit was as good everywhere: 5 x 5 torus 12.1 to 11.7
+  // ms as it is, 18.6 at 4 and 5 (layers given up); 32-site ring 4.6 as it is, 5.3 at 3.
+  float* activity;
 };
 
 // 32-bit words per plane that phases keep a string of n qubits in (P below),

@@ -122,3 +122,25 @@ def test_classes_outgrow_their_room_once_of_a_kind(lx, ly, steps):
     assert 1 <= seen[-1]["class_full"] <= 2
     assert seen[-1]["phased"] == seen[-2]["phased"] + 1 or seen[-1]["class_full"] == seen[-2]["class_full"] + 1
     assert sum(r["class_full"] == 1 for r in seen) > 1  # it is not every layer's lot
+
+
+def test_a_layer_that_grew_is_phased_again():
+    """Half of the strings, letters I and Z drawn evenly, hold a letter that a rotation
+    of one site turns.  Four such rotations, one that does not commute with them, and
+    four more multiply the strings 25 times in the first layer; the second, whose table
+    is full in these sites, is phased too."""
+    n, terms = 24, 8192
+    rng = np.random.default_rng(1)
+    z = np.unique(rng.integers(0, 1 << n, 2 * terms, dtype=np.uint64))[:terms]
+    p = pp.Propagator(n, np.zeros_like(z)[:, None], z[:, None], rng.uniform(0.5, 1.0, len(z)), symmetry=0,
+                      eps=1e-6, room_factor=10.0)
+    gates = [("x", q) for q in range(4)] + [("z", 0)] + [("x", q) for q in range(4, 8)]
+    gx = np.array([[1 << q if k == "x" else 0] for k, q in gates], dtype=np.uint64)
+    gz = np.array([[1 << q if k == "z" else 0] for k, q in gates], dtype=np.uint64)
+    th = np.full(len(gates), 0.3)
+    for _ in range(2):
+        p.apply_layer(gx[::-1].copy(), gz[::-1].copy(), th, True)
+    r, grown = pp.pp_debug_layer_routes(p.ctx), p.num_terms()[0]
+    p.close()
+    assert grown > 10 * terms
+    assert r["phased"] == 2
