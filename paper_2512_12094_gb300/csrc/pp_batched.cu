@@ -439,9 +439,13 @@ __global__ void __launch_bounds__(kBlock, W == 1 ? 3 : 2)
   __shared__ int s_ok;
   const DevTable t = *tabp;
   const unsigned first = __ldcg(&ctl->first_gate);
+  // The size at the start, from what no gate writes: a block that starts late (beside
+  // other kernels, the blocks of a cooperative launch start when there is room) would
+  // find births of the launch's first gate in the counters, where that one's slot is
+  // this one, and go its own way past the barriers.
   const int q0 = (int)((first + 2u) % 3u);
-  unsigned long long T0 = __ldcg(&ctl->base[q0]) + __ldcg(&ctl->cnt[q0]);
-  long long L0 = __ldcg(&ctl->live_base[q0]) + __ldcg(&ctl->dlt[q0]);
+  unsigned long long T0 = __ldcg(&ctl->base[q0]);
+  long long L0 = __ldcg(&ctl->live_base[q0]);
   uint64_t ox[W], oz[W];
 #pragma unroll
   for (int j = 0; j < W; ++j) {
