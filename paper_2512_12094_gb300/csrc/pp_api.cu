@@ -27,6 +27,7 @@
 #include "../../include/pp.h"
 #include "pp_internal.h"
 #include "pp_phase.h"
+#include "pp_pool_host.h"
 #include "pp_symmetry_host.h"
 
 using namespace ppk;
@@ -200,8 +201,8 @@ namespace {
 // once.  It keeps freed memory mapped (no release threshold), so tables
 // that are freed and allocated again -- a table moved when it grows, the
 // next context of a server -- reuse memory instead of mapping it anew at
-// every synchronise, as the default pool would.  The memory stays with the
-// process until it exits.
+// every synchronise, as the default pool would.  What nothing uses goes back to the
+// device at trim_pool, up to what pppool::keep leaves.
 cudaMemPool_t lib_pool() {
   static std::mutex mu;
   static std::map<int, cudaMemPool_t> pools;
@@ -221,6 +222,27 @@ cudaMemPool_t lib_pool() {
   cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
   pools[dev] = pool;
   return pool;
+}
+
+// Give back what the pool may not keep: when a context ends, and after a layer that
+// took large scratch.  The caller's stream has passed its own frees.
+void trim_pool(bool context_ends) {
+  cudaMemPool_t pool = lib_pool();
+  uint64_t reserved = 0, used = 0;
+  if (!pool || cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  const size_t unused = reserved > used ? (size_t)(reserved - used) : 0;
+  if (unused <= pppool::kKeepAlways) return;
+  size_t device_free = 0, device_total = 0;
+  if (cudaMemGetInfo(&device_free, &device_total) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  const size_t keep = pppool::keep(unused, device_free, device_total, context_ends);
+  if (keep < unused) cudaMemPoolTrimTo(pool, (size_t)used + keep);
 }
 
 // Pinned host blocks of the per-context mirrors, kept for reuse: freeing
@@ -1373,6 +1395,10 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   unsigned char* scratch = nullptr;
   auto release = [&](pp_status st) {
     dfree(c, scratch, need);
+    if (need > pppool::kKeepAlways) {
+      cudaStreamSynchronize(c->stream);
+      trim_pool(false);
+    }
     if (lent) c->give_scratch();
     return st;
   };
@@ -1766,6 +1792,7 @@ pp_status pp_destroy(pp_ctx* c) {
   dfree(c, c->d_sn, sn);
   dfree(c, c->d_sn_work, sn);
   if (c->stream) cudaStreamSynchronize(c->stream);
+  trim_pool(true);
   pinned_put(c->h_ctl, sizeof(DevCtl));
   pinned_put(c->h_out, sizeof(double) * c->B);
   pinned_put(c->h_activity, kActivityMax * sizeof(float));

@@ -43,3 +43,29 @@ def test_buckets_are_not_sized_beyond_the_strings_there_are(n):
     pp.build()
     used, tables = taken(GROWTH % n)
     assert used <= tables + (512 << 20)
+
+
+DESTROY = """
+import numpy as np, torch
+import paper_2512_12094_gb300 as pp
+torch.empty(1, device="cuda")
+rng = np.random.default_rng(0)
+m = 30000000
+x, z = (rng.integers(0, 1 << 32, (m, 1), dtype=np.uint64) for _ in range(2))
+c = rng.random(m)
+before = torch.cuda.mem_get_info()[0]
+p = pp.Propagator(32, x, z, c, symmetry=0)
+during = torch.cuda.mem_get_info()[0]
+p.close()
+print(before - during, before - torch.cuda.mem_get_info()[0])
+"""
+
+
+def test_memory_of_a_large_context_goes_back():
+    """Two tables of 120 million strings and their indexes are over 10 GB; 8 GiB of it
+    may stay mapped for the next context."""
+    import paper_2512_12094_gb300 as pp
+    pp.build()
+    during, after = taken(DESTROY)
+    assert during > 9 << 30
+    assert after <= (8 << 30) + (64 << 20)
