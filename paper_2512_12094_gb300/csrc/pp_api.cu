@@ -127,6 +127,16 @@ constexpr float kPhaseGuess = 0.09f;  // a gate's mean activity while nothing is
 constexpr int kActivityMax = 8192;
 }  // namespace
 
+// What a context has learned from its phased layers.
+struct PhasePlan {
+  double active = kPhaseActive;  // limit on the mean number of active gates of a phase
+  double room = 1.0;             // buckets per layer relative to the default sizing
+  int wait = 0;                  // layers left before phases are tried again
+  int fails = 0;                 // phased layers given up in a row
+  bool rank_bound = false;       // dense phases are cut so that no class can outgrow its room,
+  bool class_bound = false;      // and the others
+};
+
 struct pp_ctx {
   pp_config cfg{};
   int n = 0, W = 1;
@@ -181,12 +191,7 @@ struct pp_ctx {
   int64_t gates_timed = 0;
   bool index_ok = true;        // the active table's index and occupancy masks are valid
   bool phase_off = false;      // pp_tune chose the persistent kernel for this context
-  double phase_active = kPhaseActive;  // limit on the mean number of active gates of a phase
-  double phase_room = 1.0;     // buckets per layer relative to the default sizing
-  int phase_wait = 0;          // layers left before phases are tried again
-  int phase_fails = 0;         // phased layers given up in a row
-  bool rank_bound = false;     // dense phases are cut so that no class can outgrow its room,
-  bool class_bound = false;    // and the others
+  PhasePlan plan;
   int64_t routes[PP_ROUTES] = {};
   std::function<bool(size_t)> take_scratch;  // set_scratch_hooks
   std::function<void()> give_scratch;
@@ -1306,7 +1311,7 @@ PhaseSizes phase_sizes(const pp_ctx* c, size_t G, const std::vector<ppphase::Pha
   const ppphase::Workers warps = {0.5 * phase_strings_per_warp(P32), (uint64_t)c->sms * phase_warps_per_sm()};
   const ppphase::Workers blocks = c->batched ? ppphase::Workers{kRowsFill, (uint64_t)c->sms * 8}
                                              : ppphase::Workers{kDenseFill, (uint64_t)c->sms * 2};
-  z.rooms = ppphase::bucket_rooms(phases, e, blocks, warps, c->phase_room);
+  z.rooms = ppphase::bucket_rooms(phases, e, blocks, warps, c->plan.room);
   z.counters = z.records = 0;
   z.most = 0;
   for (const ppphase::Room& r : z.rooms) {
@@ -1332,8 +1337,8 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   const size_t G = args.size();
   const uint64_t T = c->n_terms;
   if (T == 0) return PP_OK;
-  if (c->phase_wait > 0) {
-    c->phase_wait--;
+  if (c->plan.wait > 0) {
+    c->plan.wait--;
     return PP_OK;
   }
   std::vector<ppphase::Gen> gens(G);
@@ -1349,11 +1354,11 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   if (ent.activity.size() != G) ent.activity.assign(G, kPhaseGuess);
   const bool dense = dense_classes(c);
   ppphase::Limits lim;
-  lim.max_active = c->phase_active;
+  lim.max_active = c->plan.active;
   lim.max_bits = kPhaseBits;
   lim.triangular = dense;
-  if (c->rank_bound) lim.max_gates = kPhaseRank;
-  if (c->class_bound) {
+  if (c->plan.rank_bound) lim.max_gates = kPhaseRank;
+  if (c->plan.class_bound) {
     // bits of which a warp holds all strings; one gate more in commuting phases, whose
     // classes seldom hold half of theirs (5 x 6 torus 35.4 ms, 35.8 without)
     const int bits = 63 - __builtin_clzll((uint64_t)phase_strings_per_warp(phase_words(c->n)));
@@ -1529,7 +1534,7 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
     c->routes[PP_ROUTE_PHASED]++;
     c->routes[PP_ROUTE_MERGE_FULL]++;
     // the gates are done, in the other table; their merge is left to the index
-    c->phase_fails = 0;
+    c->plan.fails = 0;
     c->last_growth = (double)c->h_ctl->after_terms / (double)T;
     c->n_terms = c->h_ctl->n_terms;
     c->n_live = c->h_ctl->n_live;
@@ -1549,18 +1554,18 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
     // strings: then phases have no more gates, or touch no more bits, than a class has
     // room for, and it does not happen again but for classes nearly full (dense ones in
     // either case: where a warp's class is too large a block's is soon)
-    if ((why & classes) && c->rank_bound && (c->class_bound || !(why & kPhaseClassFull)))
-      c->phase_active = std::max(0.5, 0.6 * c->phase_active);
-    if (why & classes) c->rank_bound = true;
-    if (why & kPhaseClassFull) c->class_bound = true;
+    if ((why & classes) && c->plan.rank_bound && (c->plan.class_bound || !(why & kPhaseClassFull)))
+      c->plan.active = std::max(0.5, 0.6 * c->plan.active);
+    if (why & classes) c->plan.rank_bound = true;
+    if (why & kPhaseClassFull) c->plan.class_bound = true;
     if (why & kPhaseBucketFull) {
-      c->phase_room = std::min(8.0, 2.0 * c->phase_room);
-      c->phase_active = std::max(0.5, 0.8 * c->phase_active);
+      c->plan.room = std::min(8.0, 2.0 * c->plan.room);
+      c->plan.active = std::max(0.5, 0.8 * c->plan.active);
     }
-    if (why != kPhaseTableFull) c->phase_wait = std::min(32, (1 << std::min(c->phase_fails++, 5)) - 1);
+    if (why != kPhaseTableFull) c->plan.wait = std::min(32, (1 << std::min(c->plan.fails++, 5)) - 1);
     return PP_OK;
   }
-  c->phase_fails = 0;
+  c->plan.fails = 0;
   c->routes[PP_ROUTE_PHASED]++;
   if (c->cfg.profile_kernels) {
     float ms = 0.f;
@@ -1941,11 +1946,22 @@ pp_status pp_tune(pp_ctx* c, int n_gates, const pp_pauli* gates, const double* t
   const int64_t launches = c->launches, merges = c->merges, compactions = c->compactions,
                 regrows = c->regrows, stalls = c->stalls, timed = c->gates_timed;
   const double gate_ms = c->gate_ms, growth = c->last_growth;
+  const PhasePlan plan = c->plan;
+  int64_t routes[PP_ROUTES];
+  std::copy(c->routes, c->routes + PP_ROUTES, routes);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
+  bool tuned_phased = false;
   auto finish = [&](pp_status st) {
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     free_snapshot(c, snap, n0);
+    // what the trials learned of the classes holds for the layer itself
+    const PhasePlan seen = c->plan;
+    c->plan = plan;
+    c->plan.rank_bound |= seen.rank_bound;
+    c->plan.class_bound |= seen.class_bound;
+    if (tuned_phased) c->plan.wait = 0;  // they ran here, and faster
+    std::copy(routes, routes + PP_ROUTES, c->routes);
     return st;
   };
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
@@ -1988,6 +2004,7 @@ pp_status pp_tune(pp_ctx* c, int n_gates, const pp_pauli* gates, const double* t
     }
     c->cfg.layer_kernel = tr.persistent;
     c->phase_off = !tr.phased;
+    c->plan.wait = 0;  // a phased trial is one
     c->grid_scale = tr.scale;
     if (!c->batched) {
       c->layer_threads = tr.threads;
@@ -2049,6 +2066,7 @@ pp_status pp_tune(pp_ctx* c, int n_gates, const pp_pauli* gates, const double* t
     if (rs != PP_OK) return finish(rs);
   }
   const double best_scale = best.scale;
+  tuned_phased = best.phased;
   if (upload(c, &c->d_ctl->updates, &saved, sizeof(saved)) != cudaSuccess)
     return finish(fail(PP_ERR_CUDA, "restoring statistics failed"));
   c->launches = launches;

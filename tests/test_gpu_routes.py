@@ -144,3 +144,28 @@ def test_a_layer_that_grew_is_phased_again():
     p.close()
     assert grown > 10 * terms
     assert r["phased"] == 2
+
+
+def test_tuning_leaves_the_plan_as_it_was():
+    """Tuned before a layer whose phases are given up (a class is too large): the trials
+    are not counted, and the layers after it are given up no more often, and phased no
+    less often if phases were chosen, than in a context that was not tuned."""
+    wl = pi.torus_ising(5, 6, 6, 0.4, 0.6, 0.3, 1e-4, -1, pp.sym_torus(5))
+    tuned = pp.Propagator.from_workload(wl, symmetry=wl.symmetry)
+    plain = pp.Propagator.from_workload(wl, symmetry=wl.symmetry)
+    for k, layer in enumerate(reversed(range(6))):
+        gx, gz, th = wl.circuit.gate_arrays(layer)
+        g = pp.pack_gates(gx, gz)
+        if k in (2, 4):
+            before = pp.pp_debug_layer_routes(tuned.ctx)
+            pp.pp_tune(tuned.ctx, g, th)
+            assert pp.pp_debug_layer_routes(tuned.ctx) == before
+        pp.pp_apply_layer(tuned.ctx, g, th, True)
+        pp.pp_apply_layer(plain.ctx, g, th, True)
+        assert tuned.num_terms()[0] == plain.num_terms()[0]
+    a, b = pp.pp_debug_layer_routes(tuned.ctx), pp.pp_debug_layer_routes(plain.ctx)
+    assert b["class_full"] >= 1
+    for k in GIVEN_UP:
+        assert a[k] <= b[k]
+    tuned.close()
+    plain.close()
