@@ -57,6 +57,7 @@ void ppk::set_last_error(const std::string& msg) { g_last_error = msg; }
 namespace {
 
 pp_status cuda_fail(cudaError_t e, const char* where) {
+  cudaGetLastError();  // reported here; the launch after it, in another context too, is not to find it
   std::string msg = std::string(where) + ": " + cudaGetErrorString(e);
   if (e == cudaErrorMemoryAllocation) return fail(PP_ERR_OOM, msg);
   return fail(PP_ERR_CUDA, msg);
