@@ -203,20 +203,23 @@ struct pp_ctx {
 
 namespace {
 
-// The library's stream-ordered memory pool on the current device, created
-// once.  It keeps freed memory mapped (no release threshold), so tables
+// The library's stream-ordered memory pools on the current device, created
+// once: of tables and all else a context holds, and of the scratch of phased layers.
+// They keep freed memory mapped (no release threshold), so tables
 // that are freed and allocated again -- a table moved when it grows, the
 // next context of a server -- reuse memory instead of mapping it anew at
-// every synchronise, as the default pool would.  What nothing uses goes back to the
-// device at trim_pool, up to what pppool::keep leaves.
-cudaMemPool_t lib_pool() {
+// every synchronise, as the default pool would.  The tables' memory stays with the
+// process until it exits; of the scratch's, several times theirs, what nothing uses
+// goes back to the device at trim_scratch, up to what pppool::keep leaves.
+enum Pool { kTables = 0, kScratch = 1 };
+cudaMemPool_t lib_pool(Pool which) {
   static std::mutex mu;
-  static std::map<int, cudaMemPool_t> pools;
+  static std::map<int, cudaMemPool_t> pools[2];
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
   std::lock_guard<std::mutex> lock(mu);
-  auto it = pools.find(dev);
-  if (it != pools.end()) return it->second;
+  auto it = pools[which].find(dev);
+  if (it != pools[which].end()) return it->second;
   cudaMemPoolProps props;
   memset(&props, 0, sizeof(props));
   props.allocType = cudaMemAllocationTypePinned;
@@ -226,14 +229,14 @@ cudaMemPool_t lib_pool() {
   if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) return nullptr;
   uint64_t keep = ~0ull;
   cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-  pools[dev] = pool;
+  pools[which][dev] = pool;
   return pool;
 }
 
-// Give back what the pool may not keep: when a context ends, and after a layer that
-// took large scratch.  The caller's stream has passed its own frees.
-void trim_pool(bool context_ends) {
-  cudaMemPool_t pool = lib_pool();
+// Give back what the scratch's pool may not keep: when a context ends, and after a
+// layer that took a lot.  The caller's stream has passed its own frees.
+void trim_scratch(bool context_ends) {
+  cudaMemPool_t pool = lib_pool(kScratch);
   uint64_t reserved = 0, used = 0;
   if (!pool || cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
       cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
@@ -284,7 +287,7 @@ void pinned_put(void* p, size_t bytes) {
 // before one fails as if the device were out of memory; negative = off.
 std::atomic<long long> g_fail_alloc_after{-1};
 
-pp_status dmalloc(pp_ctx* c, void** p, size_t bytes) {
+pp_status dmalloc(pp_ctx* c, void** p, size_t bytes, Pool which = kTables) {
   if (bytes == 0) bytes = 16;
   for (long long left = g_fail_alloc_after.load(); left >= 0;) {
     if (g_fail_alloc_after.compare_exchange_weak(left, left - 1)) {
@@ -295,9 +298,19 @@ pp_status dmalloc(pp_ctx* c, void** p, size_t bytes) {
       break;
     }
   }
-  cudaMemPool_t pool = lib_pool();
-  cudaError_t e = pool ? cudaMallocFromPoolAsync(p, bytes, pool, c->stream)
-                       : cudaMallocAsync(p, bytes, c->stream);
+  auto take = [&] {
+    cudaMemPool_t pool = lib_pool(which);
+    return pool ? cudaMallocFromPoolAsync(p, bytes, pool, c->stream) : cudaMallocAsync(p, bytes, c->stream);
+  };
+  cudaError_t e = take();
+  if (e == cudaErrorMemoryAllocation && which == kTables) {
+    // what the scratch's pool holds for the next layer is a table's first
+    cudaMemPool_t scratch = lib_pool(kScratch);
+    cudaStreamSynchronize(c->stream);
+    if (scratch) cudaMemPoolTrimTo(scratch, 0);
+    cudaGetLastError();
+    e = take();
+  }
   if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync");
   c->bytes += bytes;
   return PP_OK;
@@ -1401,14 +1414,14 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   unsigned char* scratch = nullptr;
   auto release = [&](pp_status st) {
     dfree(c, scratch, need);
-    if (need > pppool::kKeepAlways) {
+    if (need > pppool::kLargeScratch) {
       cudaStreamSynchronize(c->stream);
-      trim_pool(false);
+      trim_scratch(false);
     }
     if (lent) c->give_scratch();
     return st;
   };
-  if (dmalloc(c, (void**)&scratch, need) != PP_OK) {  // no room for it: the other path
+  if (dmalloc(c, (void**)&scratch, need, kScratch) != PP_OK) {  // no room for it: the other path
     cudaGetLastError();
     scratch = nullptr;
     return release(PP_OK);
@@ -1798,7 +1811,7 @@ pp_status pp_destroy(pp_ctx* c) {
   dfree(c, c->d_sn, sn);
   dfree(c, c->d_sn_work, sn);
   if (c->stream) cudaStreamSynchronize(c->stream);
-  trim_pool(true);
+  trim_scratch(true);
   pinned_put(c->h_ctl, sizeof(DevCtl));
   pinned_put(c->h_out, sizeof(double) * c->B);
   pinned_put(c->h_activity, kActivityMax * sizeof(float));

@@ -45,27 +45,31 @@ def test_buckets_are_not_sized_beyond_the_strings_there_are(n):
     assert used <= tables + (512 << 20)
 
 
-DESTROY = """
+LARGE = """
+import sys
 import numpy as np, torch
 import paper_2512_12094_gb300 as pp
 torch.empty(1, device="cuda")
 rng = np.random.default_rng(0)
-m = 30000000
-x, z = (rng.integers(0, 1 << 32, (m, 1), dtype=np.uint64) for _ in range(2))
-c = rng.random(m)
+m, n = 30000000, 32
+x, z = (rng.integers(0, 1 << n, (m, 1), dtype=np.uint64) for _ in range(2))
 before = torch.cuda.mem_get_info()[0]
-p = pp.Propagator(32, x, z, c, symmetry=0)
-during = torch.cuda.mem_get_info()[0]
+p = pp.Propagator(n, x, z, np.full(m, 1e-3), symmetry=0, eps=5e-4)
+tables = before - torch.cuda.mem_get_info()[0]
+gx = np.array([[1 << q] for q in range(8)], dtype=np.uint64)
+p.apply_layer(gx, np.zeros_like(gx), np.full(8, 0.05), True)  # births of 5e-5 are truncated
+routes = pp.pp_debug_layer_routes(p.ctx)
+during = before - torch.cuda.mem_get_info()[0]
 p.close()
-print(before - during, before - torch.cuda.mem_get_info()[0])
+print(tables, during, before - torch.cuda.mem_get_info()[0], routes["phased"])
 """
 
 
-def test_memory_of_a_large_context_goes_back():
-    """Two tables of 120 million strings and their indexes are over 10 GB; 8 GiB of it
-    may stay mapped for the next context."""
+def test_scratch_of_a_large_layer_goes_back():
+    """45 million strings expected are 64 thousand buckets of 3056 records of 32 bytes,
+    twice: 12 GB beside the tables, of which 8 GiB may stay for the next context."""
     import paper_2512_12094_gb300 as pp
     pp.build()
-    during, after = taken(DESTROY)
-    assert during > 9 << 30
-    assert after <= (8 << 30) + (64 << 20)
+    tables, during, after, phased = taken(LARGE)
+    assert phased == 1 and during > tables + (11 << 30)
+    assert after <= during - (12 << 30) + (8 << 30) + (64 << 20)
