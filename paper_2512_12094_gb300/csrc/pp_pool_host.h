@@ -1,5 +1,6 @@
-// How much memory that nothing uses the pool of the layers' scratch may keep mapped.
-// Plain C++ (no CUDA), so that the CPU tests can compile it.
+// How much memory that nothing uses the library's pool may keep mapped beyond the most
+// that tables have taken: what the scratch of layers has added to it.  Plain C++ (no
+// CUDA), so that the CPU tests can compile it.
 #pragma once
 
 #include <algorithm>

@@ -58,15 +58,23 @@ def test_reservations_without_the_scratch():
 @pytest.mark.parametrize("budget_mib", [40, 80, 160, 400])
 def test_tight_budgets_restart_nobody_more(budget_mib):
     """Eight jobs in four slots, whose tables and scratch do not all fit: no more jobs
-    start over than with the persistent kernel, and reservations stay in the budget."""
+    start over than with the persistent kernel, and reservations stay in the budget.  At
+    40 MiB who has to start over is a matter of timing, once or twice of eight jobs, with
+    a deviation below one; means of sixteen streams differ by one with a chance below
+    1 in 1000."""
     budget = budget_mib << 20
     kinds = [dict(n=32, steps=9), dict(n=24, steps=8), dict(n=40, steps=7), dict(n=16, steps=6)] * 2
-    a, most = serve([ring_job(**k) for k in kinds], 4, budget)
-    b, _ = serve([ring_job(block_threads=256, **k) for k in kinds], 4, budget)
-    assert most <= budget
-    for u, v in zip(a, b):
-        assert u["value"] == pytest.approx(v["value"], abs=1e-10)
-    assert sum(r["restarts"] for r in a) <= sum(r["restarts"] for r in b) + 1
+    streams = 16 if budget_mib < 80 else 1
+    restarts = [0, 0]
+    for _ in range(streams):
+        a, most = serve([ring_job(**k) for k in kinds], 4, budget)
+        b, _ = serve([ring_job(block_threads=256, **k) for k in kinds], 4, budget)
+        assert most <= budget
+        for u, v in zip(a, b):
+            assert u["value"] == pytest.approx(v["value"], abs=1e-10)
+        restarts[0] += sum(r["restarts"] for r in a)
+        restarts[1] += sum(r["restarts"] for r in b)
+    assert restarts[0] <= restarts[1] + streams
 
 
 def test_a_queued_job_does_not_wait_for_scratch():
