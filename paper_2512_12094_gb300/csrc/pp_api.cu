@@ -184,6 +184,7 @@ struct pp_ctx {
   bool obs_invariant = false;
   size_t bytes = 0;
   LibPool* lib = nullptr;  // of the context's device
+  size_t most_scratch = 0;  // of a layer so far
   int64_t merges = 0, compactions = 0, regrows = 0, stalls = 0;
   std::vector<GraphEntry> graphs;
   uint64_t graph_clock = 0;
@@ -1434,6 +1435,7 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
     scratch = nullptr;
     return release(PP_OK);
   }
+  c->most_scratch = std::max(c->most_scratch, need);
   PhaseAcc acc;
   acc.st = reinterpret_cast<PhaseStat*>(scratch);
   acc.delta = reinterpret_cast<long long*>(acc.st + 1);
@@ -1819,7 +1821,7 @@ pp_status pp_destroy(pp_ctx* c) {
   dfree(c, c->d_sn, sn);
   dfree(c, c->d_sn_work, sn);
   if (c->stream) cudaStreamSynchronize(c->stream);
-  trim_scratch(c->lib, true);
+  if (c->most_scratch > pppool::kSmallScratch) trim_scratch(c->lib, true);
   pinned_put(c->h_ctl, sizeof(DevCtl));
   pinned_put(c->h_out, sizeof(double) * c->B);
   pinned_put(c->h_activity, kActivityMax * sizeof(float));

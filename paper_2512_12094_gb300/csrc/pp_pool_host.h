@@ -11,9 +11,11 @@ namespace pppool {
 // Kept whatever else runs: mapping a gigabyte anew takes 0.8 ms and giving it back
 // 1.35, which small jobs one after the other would pay each time.
 constexpr size_t kKeepAlways = (size_t)1 << 30;
-// Scratch of a layer after which the pool is looked at: asking takes some 25 us, 3 % of
-// a layer of 512 columns on 10 qubits, whose scratch is 1.3 GB.
+// Scratch of a layer after which the pool is looked at, and with which a context had one
+// the end of which looks: asking takes some 25 us, 3 % of a layer of 512 columns on 10
+// qubits, whose scratch is 1.3 GB, and 1 % of a job of 45 sites and 100 columns.
 constexpr size_t kLargeScratch = (size_t)4 << 30;
+constexpr size_t kSmallScratch = (size_t)256 << 20;
 // Kept when a context ends, for the next one.
 constexpr size_t kKeepBetween = (size_t)8 << 30;
 
