@@ -131,8 +131,11 @@ typedef struct {
                               gates, a merge waiting for a claimed index slot) may last before
                               it gives up: the kernel records the failure and returns, and the
                               call reports PP_ERR_TIMEOUT; 0 = the default, 30 s (a gate over
-                              gigabytes of batched rows takes seconds).  >= 0.  Layers of a
-                              context that sets it are not applied as phases */
+                              gigabytes of batched rows takes seconds).  >= 0.  A launch's
+                              first barrier, where blocks also wait for those that find no
+                              room yet beside other contexts' kernels, has the default at
+                              least.  Layers of a context that sets it are not applied as
+                              phases */
   double room_factor;      /* headroom a layer asks for before its first gate: room for
                               2 x room_factor x (the previous layer's growth) times the
                               stored terms, and at least twice them; a layer that outgrows
@@ -298,14 +301,17 @@ pp_status pp_stats(pp_ctx* ctx, pp_stats_t* out);
 /* Raise or lower the memory budget of a context (0 = no ceiling). */
 pp_status pp_set_budget(pp_ctx* ctx, size_t mem_budget_bytes);
 
-/* Limit the kernels that apply the context's layers (by the persistent kernel one
- * cooperative launch per layer, whose blocks wait for one another at a barrier
- * between gates) to the fraction `fraction` in (0, 1] of the blocks the GPU holds at once (default
+/* Limit the context's persistent layer launches (one cooperative launch per
+ * layer whose blocks wait for one another at a barrier between gates) to the
+ * fraction `fraction` in (0, 1] of the blocks the GPU holds at once (default
  * 1).  Contexts driven from different host threads may apply layers at the
  * same time only if the fractions of those running together add up to at
  * most 1: then every launch fits beside the others.  A launch over a small
  * table uses fewer blocks than its fraction allows.  Takes effect at the
- * context's next layer.  PP_ERR_ARG for a fraction outside (0, 1]. */
+ * context's next layer.  Layers applied as phases (see layer_kernel) have no
+ * blocks that wait for one another and are not limited: a persistent launch
+ * beside them starts as they make room.  PP_ERR_ARG for a fraction outside
+ * (0, 1]. */
 pp_status pp_set_grid_fraction(pp_ctx* ctx, double fraction);
 
 /* Wait for all work queued by ctx. */

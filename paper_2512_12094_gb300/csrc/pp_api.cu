@@ -194,8 +194,7 @@ struct pp_ctx {
   double last_growth = 2.0;  // stored entries after / before the gates of the last layer
   double grid_scale = 1.0;   // blocks per launch relative to the default sizing (pp_tune)
   double index_factor = 1.5; // hash index slots per table entry of capacity (pp_tune)
-  double grid_frac = 1.0;    // a persistent layer launch takes at most this fraction of the GPU,
-  double phase_frac = 1.0;   // and a phase this one
+  double grid_frac = 1.0;    // a persistent layer launch takes at most this fraction of the GPU
   double gate_ms = 0.0;
   int64_t gates_timed = 0;
   bool index_ok = true;        // the active table's index and occupancy masks are valid
@@ -1348,7 +1347,7 @@ PhaseSizes phase_sizes(const pp_ctx* c, size_t G, const std::vector<ppphase::Pha
     // rows of the phases between, and of classes larger than shared memory
     const size_t row = (size_t)c->B * c->esize;
     z.rows = P >= 2 ? align256(c->buf[c->active].cap * row) : 0;
-    z.spill = align256(rows_launch(P32, c->B, (int)c->esize, c->sms, c->phase_frac).spill_rows * row);
+    z.spill = align256(rows_launch(P32, c->B, (int)c->esize, c->sms).spill_rows * row);
     z.bytes += z.rows + z.spill;
   }
   return z;
@@ -1411,7 +1410,10 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   const size_t need = z.bytes;
   const double est = z.est;
   const int P32 = phase_words(c->n);
-  const int warps = std::max(4, (int)std::floor(c->sms * phase_warps_per_sm() * c->phase_frac));
+  // the whole GPU whatever the context's grid fraction: their blocks wait for
+  // nothing, so launches of other contexts need no room beside them (24 served
+  // jobs: 24.5 ms, 26.2 on their fractions)
+  const int warps = c->sms * phase_warps_per_sm();
   auto al = align256;
   const size_t clear = z.clear;
   if (z.most >= (1ull << 26) || need > kPhaseBytesMax) return PP_OK;
@@ -1497,7 +1499,7 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   run(launch_phase_begin(c->stream, acc, clear, c->d_ctl, c->sms));
   const int dgrid = (int)std::min<uint64_t>((T + kBlock - 1) / kBlock, (uint64_t)c->sms * 8);
   if (c->batched) {
-    const RowsLaunch L = rows_launch(P32, c->B, (int)c->esize, c->sms, c->phase_frac);
+    const RowsLaunch L = rows_launch(P32, c->B, (int)c->esize, c->sms);
     run(launch_rows_deal(P32, dgrid, c->stream, desc_of(c, c->buf[src]), T, buckets_of(0),
                          desc(0), ent.d_args, acc));
     const void* from = c->buf[src].rows;
@@ -2306,7 +2308,7 @@ pp_status pp_stats(pp_ctx* c, pp_stats_t* out) {
 pp_status pp_set_grid_fraction(pp_ctx* c, double fraction) {
   if (!c) return fail(PP_ERR_ARG, "ctx is null");
   if (!(fraction > 0.0 && fraction <= 1.0)) return fail(PP_ERR_ARG, "fraction must be in (0, 1]");
-  ppk::set_grid_fraction(c, fraction, fraction);
+  ppk::set_grid_fraction(c, fraction);
   return PP_OK;
 }
 
@@ -2535,10 +2537,8 @@ pp_status pp_overlap_sum(int n_qubits, int symmetry, int64_t m, const uint64_t* 
 
 bool ppk::valid_group_code(int code, int n) { return valid_group(code, n); }
 
-void ppk::set_grid_fraction(pp_ctx* c, double frac, double phases) {
-  if (!c) return;
-  c->grid_frac = std::min(1.0, std::max(frac, 1e-9));
-  c->phase_frac = std::min(1.0, std::max(phases, 1e-9));
+void ppk::set_grid_fraction(pp_ctx* c, double frac) {
+  if (c) c->grid_frac = std::min(1.0, std::max(frac, 1e-9));
 }
 
 double ppk::layer_fraction_wanted(const pp_ctx* c) {

@@ -506,7 +506,7 @@ __global__ void __launch_bounds__(kBlock, W == 1 ? 3 : 2)
     if (gridDim.x == 1) {
       __threadfence();
       __syncthreads();
-    } else if (!grid_sync_b(ctl, target, s_ok, wlimit, gid)) {
+    } else if (!grid_sync_b(ctl, target, s_ok, first_barrier_limit(wlimit, e == 0), gid)) {
       return;
     }
     T0 += __ldcg(&ctl->cnt[slot]);

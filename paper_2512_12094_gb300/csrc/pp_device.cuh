@@ -64,6 +64,12 @@ __device__ __forceinline__ unsigned wait_limit_of(const DevCtl* ctl) {
   const unsigned v = *reinterpret_cast<const volatile unsigned*>(&ctl->wait_limit);
   return v ? v : kDefaultWaitLimit;
 }
+// At a launch's first barrier blocks also wait for those that have not started, for
+// want of room beside the kernels of other contexts (a phase takes the whole GPU for
+// milliseconds): that is not the wait a short limit is set for.
+__device__ __forceinline__ unsigned first_barrier_limit(unsigned limit_us, bool first) {
+  return first && limit_us < kDefaultWaitLimit ? kDefaultWaitLimit : limit_us;
+}
 
 template <int W>
 struct Key {

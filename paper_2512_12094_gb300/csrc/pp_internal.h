@@ -329,7 +329,7 @@ struct RowsLaunch {
   int threads, grid, smem_rows;  // rows of a class held in shared memory
   size_t smem, spill_rows;       // rows of scratch in global memory for larger classes
 };
-RowsLaunch rows_launch(int P, int B, int esize, int sms, double fraction = 1.0);
+RowsLaunch rows_launch(int P, int B, int esize, int sms);
 cudaError_t launch_rows_deal(int P, int grid, cudaStream_t s, const DevTable& src, uint64_t T,
                              const PhaseBuckets& out, const PhaseDesc& d,
                              const GateArgs* gates, const PhaseAcc& acc);
@@ -355,13 +355,11 @@ bool valid_group_code(int code, int n);
 }  // namespace ppk
 struct pp_ctx;
 namespace ppk {
-// Limit a context's persistent layer launches to the fraction `frac` (0, 1]
+// Limit a context's persistent layer launches (not layers applied as phases,
+// whose blocks do not wait for one another) to the fraction `frac` (0, 1]
 // of the GPU's co-resident blocks, so that contexts whose fractions add up to
-// at most 1 (the server's jobs) can run their layers at the same time; its phases
-// to the fraction `phases`.  A phase's blocks wait for nothing, but those of another
-// context's persistent launch wait at their first barrier, whose wait is limited, for
-// the ones that a phase leaves no room for.
-void set_grid_fraction(pp_ctx* c, double frac, double phases);
+// at most 1 (the server's jobs) can run their layers at the same time.
+void set_grid_fraction(pp_ctx* c, double frac);
 // The fraction of the GPU's co-resident blocks the context's next persistent
 // layer launch would use with no limit (0 when it has no persistent path).
 double layer_fraction_wanted(const pp_ctx* c);

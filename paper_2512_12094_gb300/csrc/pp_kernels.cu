@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(NT, NT == 1024 ? 1 : ((W == 1) ? 4 : 2))
       // fence and the block barrier, are all the next gate depends on
       __threadfence();
       __syncthreads();
-    } else if (!grid_sync(ctl, target, s_ok, wlimit, gid)) {
+    } else if (!grid_sync(ctl, target, s_ok, first_barrier_limit(wlimit, e == 0), gid)) {
       return;
     }
     T0 += __ldcg(&ctl->cnt[slot]);

@@ -387,7 +387,7 @@ cudaError_t launch_rows_pt(const RowsLaunch& L, cudaStream_t s, const PhaseBucke
 
 }  // namespace
 
-RowsLaunch rows_launch(int P, int B, int esize, int sms, double fraction) {
+RowsLaunch rows_launch(int P, int B, int esize, int sms) {
   RowsLaunch L;
   L.threads = std::min(256, std::max(64, (B + 31) / 32 * 32));
   const size_t fixed = ((P == 1 ? sizeof(RowsSmem<1>) : sizeof(RowsSmem<2>)) + 15) / 16 * 16;
@@ -397,7 +397,7 @@ RowsLaunch rows_launch(int P, int B, int esize, int sms, double fraction) {
   L.smem_rows = (int)std::min<size_t>(kRMembers, (room - fixed) / row);
   L.smem = fixed + (size_t)L.smem_rows * row;
   const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(8, 226 * 1024 / (L.smem + 1024)));
-  L.grid = std::max(1, (int)(sms * per_sm * fraction));
+  L.grid = sms * per_sm;
   L.spill_rows = (size_t)L.grid * kRMembers;
   return L;
 }

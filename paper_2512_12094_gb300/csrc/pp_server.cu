@@ -97,8 +97,6 @@ struct pp_server {
   std::deque<std::unique_ptr<Job>> queue;
   std::map<uint64_t, Done> results;
   int64_t running = 0, completed = 0;
-  int64_t limited = 0;  // running jobs that set a wait limit
-  int64_t wide = 0;     // layers in hand whose phases may take the whole GPU
   int units_free = 0;  // share units of the GPU's co-resident blocks not held by a layer
   ppadm::CostModel cost;  // predicted run times of queued jobs (admission order)
   std::mutex mu;
@@ -184,27 +182,6 @@ void release_units(pp_server* s, int units) {
   std::lock_guard<std::mutex> lock(s->mu);
   s->units_free += units;
   s->cv_work.notify_all();
-}
-
-// Before a layer: may its phases take the whole GPU and not only the job's share (24
-// served jobs: 24.5 ms, 26.2 on their shares)?  Not while a job with a wait limit of its
-// own runs, whose barriers would wait for room beside them; the layers of such a job
-// wait for those that already may.
-bool begin_layer(pp_server* s, const Job& j) {
-  std::unique_lock<std::mutex> lock(s->mu);
-  if (j.cfg.wait_limit > 0) {
-    s->cv_work.wait(lock, [&] { return s->wide == 0; });
-    return false;
-  }
-  if (s->limited > 0) return false;
-  s->wide++;
-  return true;
-}
-
-void end_layer(pp_server* s, bool wide) {
-  if (!wide) return;
-  std::lock_guard<std::mutex> lock(s->mu);
-  if (--s->wide == 0 && s->limited > 0) s->cv_work.notify_all();
 }
 
 enum class Grow { kGranted, kNever, kGiveBack };
@@ -324,13 +301,10 @@ pp_status run_job(pp_server* s, Job& j, cudaStream_t stream, pp_job_result& r, b
       // any wait for memory, so no job waits for memory while holding units
       // another job needs in order to finish.
       const double wanted = ppk::layer_fraction_wanted(ctx);
-      const bool wide = begin_layer(s, j);
       const int units = wanted > 0.0 ? acquire_units(s, wanted) : 0;
-      const double share = units > 0 ? (double)units / ppadm::kShareUnits : 1.0;
-      ppk::set_grid_fraction(ctx, share, wide ? 1.0 : share);
+      if (units > 0) ppk::set_grid_fraction(ctx, (double)units / ppadm::kShareUnits);
       st = pp_apply_layer(ctx, (int)j.gates.size(), j.gates.data(), j.theta.data(), j.boundary);
       if (units > 0) release_units(s, units);
-      end_layer(s, wide);
       if (st != PP_ERR_CAPACITY || !grow_or_stop(st)) break;
     }
   }
@@ -360,7 +334,6 @@ void worker_main(pp_server* s) {
       if (!j) break;  // stopping and nothing left that fits
       s->reserved += j->reserve;
       s->running++;
-      s->limited += j->cfg.wait_limit > 0;
     }
     if (!j->started) {
       j->t_start = Clock::now();
@@ -379,7 +352,6 @@ void worker_main(pp_server* s) {
     std::unique_lock<std::mutex> lock(s->mu);
     s->reserved -= j->reserve;  // every granted increase was added to `reserved`
     s->running--;
-    s->limited -= j->cfg.wait_limit > 0;
     if (give_back) {
       j->reserve = j->want_next;
       j->restarts++;
