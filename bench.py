@@ -11,9 +11,11 @@ weight <= 10, FP64.  It is propagated twice, plain and Z_32-merged, and
 Prints one JSON line (rank 0).  ``value`` is measured with the observable
 already in device memory; ``e2e`` goes through the host-buffer C-ABI calls
 (pp_create from host arrays, pp_expect back to the host).  Both timed regions
-run the job without instrumentation.  ``roofline`` is for the layer kernel,
-timed with CUDA events around every layer kernel on the context's stream in a
-separate pass of the same jobs.  ``cpu_baseline`` times the CPU
+run the job without instrumentation.  ``roofline`` is for the kernels that
+apply a layer's gates, timed with CUDA events around them on the context's stream in
+a separate pass of the same jobs; its bytes are those of a pass over the table per
+gate, which layers applied as phases do without, and ``fp64`` beside it has what
+those are bound by.  ``cpu_baseline`` times the CPU
 oracle on a bounded prefix of the same workload.  ``served`` (one GPU only)
 is the serving part of the metric: a scaled Poisson stream of 300 jobs
 through pp_submit after the main job, with jobs/s and latency p50/p99
@@ -55,6 +57,28 @@ def algorithmic_bytes(updates, skipped_updates, anticommuting):
     anticommuting term.  Updates in gates the occupancy test skipped move no
     bytes (every string commutes with the gate and nothing is read)."""
     return KEY_BYTES * (updates - skipped_updates) + BYTES_PER_ANTICOMMUTING * anticommuting
+
+
+# Rotations: two products and a sum for each member of a pair, and what an SM's
+# FP64 pipe takes, two a cycle.
+FLOPS_PER_ANTICOMMUTING = 3
+FP64_PER_CYCLE_AND_SM = 2
+SMS = 152
+
+
+def fp64_summary(anticommuting, gate_ms, sm_mhz):
+    """Products and sums of the rotations against the FP64 pipes at the clock seen
+    (dense_phase_kernel<1>: the pipe is busy half of the time, the rest is barriers;
+    profiles/phase_kernels_ring32_zn.md)."""
+    if not gate_ms or not sm_mhz:
+        return None
+    peak = FP64_PER_CYCLE_AND_SM * SMS * sm_mhz * 1e6
+    rate = FLOPS_PER_ANTICOMMUTING * anticommuting / (gate_ms / 1e3)
+    return {"achieved": rate / 1e9, "peak": peak / 1e9, "unit": "G products or sums/s", "frac": rate / peak,
+            "model": "two products and a sum per live anticommuting term; two a cycle and SM at the "
+                     "median clock under load"}
+
+
 # DRAM bytes (read + write) per algorithmic byte of layer_kernel<1>, from one
 # ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of the last layer
 # of the Z_32-merged job, taken with the kernel sources whose digest is
@@ -437,22 +461,28 @@ def bench_ours(args):
                      "frac": (achieved / hbm) if achieved else None,
                      "traffic": traffic_per_launch(bytes_alg / max(gate_n, 1)),
                      "traffic_basis": "ncu DRAM bytes per algorithmic byte of the last layer "
-                                      "of the Z_32 job x this run's average launch; null when "
-                                      "the kernel sources differ from the captured ones",
+                                      "of the Z_32 job by layer_kernel<1> x this run's average "
+                                      "launch; null when the kernel sources differ from the "
+                                      "captured ones (dense_phase_kernel<1>: 124 MB a launch on "
+                                      "1.6 to 3 million strings, 7 % of DRAM)",
                      "kernel": "layers as phases (dense_phase_kernel<1>) and layer_kernel<1>",
+                     "fp64": fp64_summary(ac, gate_ms, (clk or {}).get("sm_mhz")),
                      "block_threads": stats[-1]["block_threads"],
                      "peak_kind": peak_kind,
                      "peak_nominal": HBM_NOMINAL_GBS,
                      "frac_nominal": (achieved / HBM_NOMINAL_GBS) if achieved else None,
                      "bytes_model": "16 B key per live term entering a scanned gate + 64 B per "
                                     "live anticommuting term (gates skipped by the occupancy "
-                                    "test move no bytes)",
+                                    "test move no bytes): a pass over the table per gate.  A phase "
+                                    "moves two 32 B records a string for up to 32 gates, so "
+                                    "achieved is not what passes DRAM",
                      "skipped_updates_fraction": (skipped / pupd) if pupd else None,
                      "gates_skipped_per_job": gates_skipped / max(args.steps, 1),
                      "avg_launch_us": 1e3 * gate_ms / max(gate_n, 1),
                      "algorithmic_bytes_per_launch": bytes_alg / max(gate_n, 1),
-                     "timing": "CUDA events around every layer kernel, in a pass of the "
-                               "same jobs after the timed regions"},
+                     "timing": "CUDA events around the kernels that apply a layer's gates (all "
+                               "phases of a layer, or a layer_kernel), in a pass of the same "
+                               "jobs after the timed regions"},
         "clocks": clk,
         "cpu_baseline": cpu,
         "served": served,

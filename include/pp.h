@@ -357,8 +357,10 @@ pp_status pp_canonical_keys(int n_qubits, int symmetry, int64_t m, const uint64_
  * to its representative under `symmetry` (PP_SYM_NONE: identity), i.e. the
  * merge loop of Algorithms 2 and 3.  Writes the distinct strings and their
  * FP64 sums to keys_out [m][2W], coef_out [m] in unspecified order and the
- * count to *m_out (host pointer; the call synchronises the stream).  Uses a
- * temporary device hash table obtained with cudaMallocAsync on `stream`. */
+ * count to *m_out (host pointer; the call synchronises the stream).  Uses
+ * temporary buckets of the strings or a hash table (S_n, lists with many equal
+ * strings, outputs over the inputs, no memory for the buckets), obtained with
+ * cudaMallocAsync on `stream`. */
 pp_status pp_merge_terms(int n_qubits, int symmetry, int64_t m, const uint64_t* keys_in,
                          const double* coef_in, uint64_t* keys_out, double* coef_out,
                          int64_t* m_out, void* stream);

@@ -1295,19 +1295,29 @@ bool phases_allowed(const pp_ctx* c) {
 //
 // Rule: at least kPhaseMinGates gates that touch a string per phase, since a phase
 // costs two passes over the table and two launches whatever it holds, and a
-// pass per gate costs one and a barrier.
+// pass per gate costs one and a barrier.  (2, 3, 4 and 6: ring of 101 sites 2.26, 2.28,
+// 2.32 and 2.59 ms, all-to-all 64 sites under S_n 11.3, 11.3, 11.7 and 11.4.)
 constexpr int kPhaseMinGates = 3;
-constexpr int kPhaseMax = 64;       // phases of a layer
+// Phases of a layer.  Only unmerged all-to-all layers pass it, with 510 on 64 sites: ten
+// of them 357 ms on the persistent kernel and 282 as phases, so the line could lie
+// higher; what so many launches cost where the tables stay small is not measured.
+constexpr int kPhaseMax = 64;
 // Strings of the input table from which a phased layer's merge goes by buckets.
 // Layers of the 32-site ring take the same with 1024, 8192 and 65536 (16.9 to 17.2
 // ms for 20 of them; 18.5 with the index at every size); below, the merge costs a
 // few launches either way, and the index is of use to a layer the persistent
 // kernel applies next.
 constexpr uint64_t kMergeTerms = 1024;
-constexpr double kRowsFill = 8.0;    // of rows
+// Rows of a bucket in the expected table (4, 8, 16, 32: 64 sites and 256 FP64 columns
+// 3.85, 3.62, 3.59 and 3.53 ms).
+constexpr double kRowsFill = 8.0;
 constexpr double kDenseFill = 700.0; // strings of a bucket in the expected table, dense classes
-constexpr int kPhaseBits = 10;      // key bits a run that does not commute may touch
-
+// Key bits a run that does not commute may touch (8 to 12: all-to-all 64 sites under S_n
+// 11.7, 11.8, 11.4, 11.6 and 11.3 ms, 24 served jobs 17.0, 17.5, 16.9, 17.3 and 18.8).
+constexpr int kPhaseBits = 10;
+// Scratch of a layer: a bound to what a call may take beside its tables, a quarter of
+// this chip's memory and some 230 million strings, not a line between two speeds; larger
+// layers are the persistent kernel's, as all were.
 constexpr size_t kPhaseBytesMax = (size_t)64 << 30;
 
 size_t align256(size_t b) { return (b + 255) / 256 * 256; }

@@ -250,8 +250,8 @@ __device__ __forceinline__ T warp_sum(T v) {
 
 // ----------------------------------------------------------- gate kernel
 
-template <int W, class Gate>
-__device__ __forceinline__ int sigma_of(const Gate& g, const Key<W>& q) {
+template <int W>
+__device__ __forceinline__ int sigma_of(const GateArgs& g, const Key<W>& q) {
   // P Q = i^E R with E = sum_sites px pz + qx qz + 2 pz qx - (px^qx)(pz^qz)
   // (P = i^{px pz} X^px Z^pz per site); i P Q = i^{E+1} R and E+1 is even.
   int e = g.pyy;
@@ -282,22 +282,7 @@ __device__ __forceinline__ double with_sign(double c, bool negate) {
 
 // -------------------------------------------------- canonicalisation
 
-// Digit word of Def. "Lowest integer representation": bit 2q = x_q ^ z_q,
-// bit 2q+1 = z_q, so the 2-bit digit of qubit q is I=0, X=1, Y=2, Z=3.
-__device__ __forceinline__ uint64_t spread32(uint32_t a) {
-  uint64_t x = a;
-  x = (x | (x << 16)) & 0x0000FFFF0000FFFFull;
-  x = (x | (x << 8)) & 0x00FF00FF00FF00FFull;
-  x = (x | (x << 4)) & 0x0F0F0F0F0F0F0F0Full;
-  x = (x | (x << 2)) & 0x3333333333333333ull;
-  x = (x | (x << 1)) & 0x5555555555555555ull;
-  return x;
-}
-
-__device__ __forceinline__ uint64_t digits32(uint32_t x, uint32_t z) {
-  return spread32(x ^ z) | (spread32(z) << 1);
-}
-
+// Def. "Lowest integer representation": the digit of qubit q is I=0, X=1, Y=2, Z=3.
 template <int W>
 __device__ __forceinline__ int digit_at(const Key<W>& k, int q) {
   const int xb = (int)((k.x(q >> 6) >> (q & 63)) & 1ull);
@@ -483,8 +468,9 @@ __device__ __forceinline__ uint64_t zn_after_longest_runs(uint64_t v, int n, uin
 // instructions: four million strings of 64 sites in 54, 60, 63 and 68 us at
 // weights 4, 8, 12 and 32, where walking gaps took 61, 95 and 127 us and shrinking
 // masks 72 at 32; at weight 48 shrinking takes 63 and doubling 70, which is the
-// reason for the half (at 32 sites they meet at weight 18).  Otherwise they are found in
-// one of two ways, both giving every longest run:
+// reason for the half (at 32 sites they meet at weight 18).  Of strings of weight 2
+// alone, doubling takes 50 us and gaps 46.  Otherwise they are found in one of two
+// ways, both giving every longest run:
 //  * few sites differ from d (a low-weight string, d = I): walk the gaps
 //    between consecutive such sites, cyclically; a gap before site s is a
 //    run ending just before s, so j = s;

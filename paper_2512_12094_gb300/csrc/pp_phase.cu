@@ -12,8 +12,8 @@
 // Why: one pass per gate costs a grid barrier, dependent L2 loads and a births
 // flush whatever the table (9 us a gate at 10^5 strings), and three random
 // 32-byte HBM sectors per anticommuting string on large tables.  A phase costs
-// two passes over the table (24 bytes a string in and out for n <= 32, half of
-// it scattered) and the instructions of the gates, which are what bounds it.
+// two passes over the table (a record of 32 bytes a string in and out up to 64 sites,
+// half of it scattered) and the instructions of the gates, which are what bounds it.
 //
 // Why a warp per bucket: only some 15 % of a bucket's strings anticommute with
 // a gate.  A warp needs 200 strings or more to fill its lanes with them; blocks
@@ -38,8 +38,7 @@ constexpr int kPosBits = 11;    // of an index slot: position + 1; a tag above i
 constexpr unsigned kPosMask = (1u << kPosBits) - 1u;
 // Strings are kept in P 32-bit words per plane: one for n <= 32 (half the
 // shared memory and bucket traffic of the 64-bit words of the table).
-// C: strings of a warp; kSlots: index slots, at most 3/4 full; both are divided
-// among the warp's warps.
+// C: strings of a warp; kSlots: its index slots, at most 3/4 full.
 template <int P>
 struct PhaseDims {
   static constexpr int C = P == 1 ? 736 : (P == 2 ? 480 : (P == 4 ? 320 : (P == 6 ? 224 : 192)));
@@ -523,7 +522,8 @@ __global__ void __launch_bounds__(kPT, kPBlocks)
 constexpr int kDT = 512;       // threads of a dense block
 constexpr int kDStrings = 1024;
 constexpr int kDSlots = 2048;  // coefficients of all classes of a part
-constexpr int kDOrder = 4096;  // (class, active gate) entries
+// (class, active gate) entries: r for a class of 2^(r - 1) >= r pairs
+constexpr int kDOrder = kDSlots / 2;
 constexpr int kDTable = 2048;  // hash slots of the class lookup
 struct DClass {
   uint16_t off, pairs;  // first slot, first pair
@@ -711,7 +711,7 @@ __global__ void __launch_bounds__(kDT, 2)
           const int rank = __popc(act), size = 1 << rank;
           const int off = atomicAdd(&S.slots, size), od = rank ? atomicAdd(&S.orders, rank) : 0;
           const int pr = rank ? atomicAdd(&S.bin[rank], size / 2) : 0;
-          if (off + size > kDSlots || od + rank > kDOrder) continue;  // seen below
+          if (off + size > kDSlots) continue;  // seen below
           DClass C;
           C.off = (uint16_t)off;
           C.pairs = (uint16_t)pr;
@@ -733,7 +733,7 @@ __global__ void __launch_bounds__(kDT, 2)
         }
       }
       __syncthreads();
-      const bool fits = laid && S.slots <= kDSlots && S.orders <= kDOrder;
+      const bool fits = laid && S.slots <= kDSlots;
       if (!fits) {  // uniform
         if (S.bad || ++s > kMaxSplit) {
           fail |= S.bad ? kPhaseRankFull : kPhaseClassFull;
@@ -963,7 +963,7 @@ cudaError_t launch_dense_p(int warps, cudaStream_t s, const PhaseBuckets& in, co
   static SmemLimit limit;
   const cudaError_t e = limit.raise(dense_phase_kernel<P>, sizeof(DenseSmem<P>));
   if (e != cudaSuccess) return e;
-  // two blocks of 8 warps per SM where phase_kernel has three of 4
+  // two blocks of 16 warps per SM where phase_kernel has three of 4
   const int grid = std::max(1, warps / (kPW * kPBlocks) * 2);
   dense_phase_kernel<P><<<grid, kDT, sizeof(DenseSmem<P>), s>>>(in, out, d, next, gates, rule,
                                                                 dense, ctl, acc);

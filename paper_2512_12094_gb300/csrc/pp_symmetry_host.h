@@ -15,9 +15,8 @@
 
 namespace ppsym {
 
-inline void permute_string(const uint64_t* x, const uint64_t* z, int n, int W,
+inline void permute_string(const uint64_t* x, const uint64_t* z, int W,
                            const std::vector<int>& to, uint64_t* ox, uint64_t* oz) {
-  (void)n;
   for (int j = 0; j < W; ++j) ox[j] = oz[j] = 0;
   for (int j = 0; j < W; ++j)  // the sites that hold a letter
     for (uint64_t m = x[j] | z[j]; m; m &= m - 1) {
@@ -120,7 +119,7 @@ inline bool multiset_invariant(int group, int n, int W, const uint64_t* keys, co
   for (const auto& g : gens) {
     for (size_t i = 0; i < m; ++i) {
       const uint64_t* k = keys + i * K;
-      permute_string(k, k + W, n, W, g, &img[i * K], &img[i * K + W]);
+      permute_string(k, k + W, W, g, &img[i * K], &img[i * K + W]);
     }
     const std::vector<uint32_t> at = key_order(img.data(), m, K);
     const std::vector<double> v = sorted_values(img.data(), at);
