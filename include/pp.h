@@ -156,8 +156,9 @@ typedef struct {
   int64_t compactions;
   int64_t regrows;
   size_t device_bytes;     /* device memory currently held by the context (a call's own
-                              scratch, such as the buckets of a layer's phases, is given
-                              back before it returns) */
+                              scratch, such as the buckets of a layer's phases, goes back
+                              to the library's memory pool before it returns, and from
+                              there to the device if the pool may not keep it) */
   double anticommuting_terms; /* sum over applied gates of live terms anticommuting with P */
   int64_t kernel_launches; /* kernels launched by the context (graph nodes included) */
   double gate_kernel_ms;   /* with profile_kernels: summed duration of the kernels that applied
@@ -440,7 +441,9 @@ typedef struct {
  * finished jobs on the job's layers, gates per layer, threshold, noise, n and
  * group) less one natural-log unit per 10 s waited, so short jobs do not
  * wait behind long ones and every job reaches the front; their kernels
- * overlap on the device.  A running job waiting for a larger reservation is
+ * overlap on the device.  The scratch with which a layer runs as phases is
+ * lent on top of the reservation for that layer, if neither a running job nor
+ * a queued one needs the memory.  A running job waiting for a larger reservation is
  * served before any queued job is admitted, and a queued job that jobs after
  * it in that order have passed 8 times is not passed again.
  * default_job_bytes: reservation of jobs that name none; 0 = estimate each
