@@ -135,7 +135,8 @@ struct PhasePlan {
   int wait = 0;                  // layers left before phases are tried again
   int fails = 0;                 // phased layers given up in a row
   bool rank_bound = false;       // dense phases are cut so that no class can outgrow its room,
-  bool class_bound = false;      // and the others
+  bool plain_bound = false;      // other commuting phases,
+  bool class_bound = false;      // and those that do not commute
 };
 
 // The memory pool of a device (lib_pool).
@@ -1390,13 +1391,11 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   lim.max_bits = kPhaseBits;
   lim.triangular = dense;
   if (c->plan.rank_bound) lim.max_gates = kPhaseRank;
-  if (c->plan.class_bound) {
-    // bits of which a warp holds all strings; one gate more in commuting phases, whose
-    // classes seldom hold half of theirs (5 x 6 torus 35.4 ms, 35.8 without)
-    const int bits = 63 - __builtin_clzll((uint64_t)phase_strings_per_warp(phase_words(c->n)));
-    lim.max_plain = bits + 1;
-    lim.max_bits = std::min(kPhaseBits, bits);
-  }
+  // bits of which a warp holds all strings; one gate more in commuting phases, whose
+  // classes seldom hold half of theirs (5 x 6 torus 35.1 ms, 35.8 without)
+  const int bits = 63 - __builtin_clzll((uint64_t)phase_strings_per_warp(phase_words(c->n)));
+  if (c->plan.plain_bound) lim.max_plain = bits + 1;
+  if (c->plan.class_bound) lim.max_bits = std::min(kPhaseBits, bits);
   lim.max_phases = std::min<size_t>(kPhaseMax, n_touch / kPhaseMinGates);
   std::vector<ppphase::Phase> phases = ppphase::plan(gens, c->W, touch.data(), ent.activity.data(), lim);
   if (phases.size() > lim.max_phases) {
@@ -1582,18 +1581,21 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   if (const unsigned why = c->h_ctl->stall) {
     // given up: the input table is whole (its index may not be).  Next time
     // with finer phases or more buckets, and after ever longer waits.
-    const unsigned classes = kPhaseClassFull | kPhaseRankFull;
+    const unsigned classes = kPhaseClassFull | kPhasePlainFull | kPhaseRankFull;
     c->routes[(why & classes)            ? PP_ROUTE_CLASS_FULL
               : (why & kPhaseBucketFull) ? PP_ROUTE_BUCKET_FULL
                                          : PP_ROUTE_TABLE_FULL]++;
     // a class of more active gates than its room (a star of bonds), or of more
-    // strings: then phases have no more gates, or touch no more bits, than a class has
-    // room for, and it does not happen again but for classes nearly full (dense ones in
-    // either case: where a warp's class is too large a block's is soon)
-    if ((why & classes) && c->plan.rank_bound && (c->plan.class_bound || !(why & kPhaseClassFull)))
-      c->plan.active = std::max(0.5, 0.6 * c->plan.active);
-    if (why & classes) c->plan.rank_bound = true;
-    if (why & kPhaseClassFull) c->plan.class_bound = true;
+    // strings: then phases of its kind have no more gates, or touch no more bits, than a
+    // class has room for, and it does not happen again but for classes nearly full
+    // (dense ones in any case: where a warp's class is too large a block's is soon)
+    PhasePlan& p = c->plan;
+    if ((why & classes) && p.rank_bound && (p.plain_bound || !(why & kPhasePlainFull)) &&
+        (p.class_bound || !(why & kPhaseClassFull)))
+      p.active = std::max(0.5, 0.6 * p.active);
+    if (why & classes) p.rank_bound = true;
+    if (why & kPhasePlainFull) p.plain_bound = true;
+    if (why & kPhaseClassFull) p.class_bound = true;
     if (why & kPhaseBucketFull) {
       c->plan.room = std::min(8.0, 2.0 * c->plan.room);
       c->plan.active = std::max(0.5, 0.8 * c->plan.active);
@@ -1995,6 +1997,7 @@ pp_status pp_tune(pp_ctx* c, int n_gates, const pp_pauli* gates, const double* t
     const PhasePlan seen = c->plan;
     c->plan = plan;
     c->plan.rank_bound |= seen.rank_bound;
+    c->plan.plain_bound |= seen.plain_bound;
     c->plan.class_bound |= seen.class_bound;
     if (tuned_phased) c->plan.wait = 0;  // they ran here, and faster
     std::copy(routes, routes + PP_ROUTES, c->routes);

@@ -255,6 +255,7 @@ enum : unsigned {
   kPhaseClassFull = 2u,  // one class outgrew a warp's shared memory
   kPhaseTableFull = 4u,  // the destination table
   kPhaseRankFull = 16u,  // a dense class has more than kPhaseRank active gates
+  kPhasePlainFull = 32u,  // kPhaseClassFull of a commuting phase
 };
 
 struct alignas(16) PhaseStat {

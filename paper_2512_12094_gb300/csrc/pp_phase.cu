@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(kPT, kPBlocks)
     if (cnt) {
       if (!ok) {
         if (++s > kMaxSplit) {
-          fail |= kPhaseClassFull;
+          fail |= d.commuting ? kPhasePlainFull : kPhaseClassFull;
           cnt = 0;  // given up
         }
       } else {
