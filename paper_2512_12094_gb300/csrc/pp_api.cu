@@ -135,7 +135,8 @@ struct PhasePlan {
   int wait = 0;                  // layers left before phases are tried again
   int fails = 0;                 // phased layers given up in a row
   bool rank_bound = false;       // dense phases are cut so that no class can outgrow its room,
-  bool plain_bound = false;      // other commuting phases,
+  bool plain_finer = false;      // other commuting phases with fewer active gates,
+  bool plain_bound = false;      // and so too,
   bool class_bound = false;      // and those that do not commute
 };
 
@@ -1392,7 +1393,7 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
   lim.triangular = dense;
   if (c->plan.rank_bound) lim.max_gates = kPhaseRank;
   // bits of which a warp holds all strings; one gate more in commuting phases, whose
-  // classes seldom hold half of theirs (5 x 6 torus 35.1 ms, 35.8 without)
+  // classes seldom hold half of theirs (5 x 6 torus 35.4 ms, 35.8 without)
   const int bits = 63 - __builtin_clzll((uint64_t)phase_strings_per_warp(phase_words(c->n)));
   if (c->plan.plain_bound) lim.max_plain = bits + 1;
   if (c->plan.class_bound) lim.max_bits = std::min(kPhaseBits, bits);
@@ -1588,13 +1589,21 @@ pp_status apply_layer_phased(pp_ctx* c, ArgsEntry& ent, const std::vector<GateAr
     // a class of more active gates than its room (a star of bonds), or of more
     // strings: then phases of its kind have no more gates, or touch no more bits, than a
     // class has room for, and it does not happen again but for classes nearly full
-    // (dense ones in any case: where a warp's class is too large a block's is soon)
+    // (dense ones in any case: where a warp's class is too large a block's is soon).
+    // Where none are dense, commuting phases first have fewer active gates: the layers
+    // of a ring of 100 sites, whose gates are active on few strings each, take 0.6 ms
+    // so and 0.7 with nine gates a phase.
     PhasePlan& p = c->plan;
     if ((why & classes) && p.rank_bound && (p.plain_bound || !(why & kPhasePlainFull)) &&
         (p.class_bound || !(why & kPhaseClassFull)))
       p.active = std::max(0.5, 0.6 * p.active);
     if (why & classes) p.rank_bound = true;
-    if (why & kPhasePlainFull) p.plain_bound = true;
+    if ((why & kPhasePlainFull) && (dense || p.plain_finer)) {
+      p.plain_bound = true;
+    } else if (why & kPhasePlainFull) {
+      p.plain_finer = true;
+      p.active = std::max(0.5, 0.6 * p.active);
+    }
     if (why & kPhaseClassFull) p.class_bound = true;
     if (why & kPhaseBucketFull) {
       c->plan.room = std::min(8.0, 2.0 * c->plan.room);

@@ -34,6 +34,10 @@ namespace {
 
 constexpr int kPW = 4;          // warps of a phase block
 constexpr int kPT = 32 * kPW;
+// A warp's bucket is cut into at most 2^kWarpSplit parts (a class that is too large
+// among small ones is found by cutting on: 85 us a bit at 4 words, 16 bits 2.3 ms of a
+// layer given up and 10 bits 1.7)
+constexpr int kWarpSplit = 10;
 constexpr int kPosBits = 11;    // of an index slot: position + 1; a tag above it
 constexpr unsigned kPosMask = (1u << kPosBits) - 1u;
 // Strings are kept in P 32-bit words per plane: one for n <= 32 (half the
@@ -421,7 +425,7 @@ __global__ void __launch_bounds__(kPT, kPBlocks)
     __syncwarp();
     const bool too_many = n > C;
     // one class, which no further bit of its hash divides
-    if (too_many && __reduce_and_sync(kFull, all) == __reduce_or_sync(kFull, any)) s = kMaxSplit;
+    if (too_many && __reduce_and_sync(kFull, all) == __reduce_or_sync(kFull, any)) s = kWarpSplit;
     n = phase_gates<P>(S, B.gate, d, rule, too_many ? 0 : n, uni);
     if (too_many) n = -1;
     const bool ok = n >= 0;
@@ -473,7 +477,7 @@ __global__ void __launch_bounds__(kPT, kPBlocks)
     }
     if (cnt) {
       if (!ok) {
-        if (++s > kMaxSplit) {
+        if (++s > kWarpSplit) {
           fail |= d.commuting ? kPhasePlainFull : kPhaseClassFull;
           cnt = 0;  // given up
         }

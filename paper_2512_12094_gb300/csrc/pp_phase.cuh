@@ -7,7 +7,7 @@
 namespace ppk {
 namespace {
 
-// A bucket is cut into at most 2^kMaxSplit parts.  Two classes that only just fit a
+// A block's bucket is cut into at most 2^kMaxSplit parts.  Two classes that only just fit a
 // part each must not meet in one: with 10 bits they did in some bucket of thousands.
 constexpr int kMaxSplit = 16;
 
